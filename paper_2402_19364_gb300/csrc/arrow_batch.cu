@@ -242,7 +242,7 @@ int arrow_batch_spmm(arrow_batch B, const void* const* X, void* const* Y, const 
             const arrow_handle_s* h = B->hs[m];
             const DeviceData& d = h->dev;
             MatDesc md{};
-            md.rowptr = d.rowptr; md.col = d.col; md.val = d.val; md.tile_row = d.tile_row; md.tile_ent = d.tile_ent;
+            md.rowptr = d.rowptr; md.row_desc = d.row_desc; md.col = d.col; md.val = d.val; md.tile_row = d.tile_row; md.tile_ent = d.tile_ent;
             md.lcol = d.lcol; md.lval = d.lval; md.seg_begin = d.seg_begin; md.seg_end = d.seg_end;
             md.long_rows = d.long_rows; md.long_segptr = d.long_segptr; md.perm0 = d.perm0; md.iperm0 = d.iperm0;
             md.x_user = X[m]; md.y_user = Y[m];

@@ -77,6 +77,7 @@ struct DeviceData {
     void* val = nullptr;            // [nnz_short] values, value_dtype
     int32_t* tile_row = nullptr;    // [n_tiles+1] first row of each tile
     int32_t* tile_ent = nullptr;    // [n_tiles+1] first entry of each tile
+    uint32_t* row_desc = nullptr;   // [n] per tile: its rows by decreasing length (row_desc_pack)
     int32_t* lcol = nullptr;        // [nnz_long] entries of the split rows
     void* lval = nullptr;           // [nnz_long]
     int32_t* perm0 = nullptr;       // [n]  vertex -> pi_0 position

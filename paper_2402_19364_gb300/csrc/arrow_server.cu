@@ -330,7 +330,7 @@ static int server_step(arrow_server_s* S, void* stream, int32_t* active_out) {
         const arrow_handle_s* h = r.h;
         const DeviceData& d = h->dev;
         MatDesc md{};
-        md.rowptr = d.rowptr; md.col = d.col; md.val = d.val; md.tile_row = d.tile_row; md.tile_ent = d.tile_ent;
+        md.rowptr = d.rowptr; md.row_desc = d.row_desc; md.col = d.col; md.val = d.val; md.tile_row = d.tile_row; md.tile_ent = d.tile_ent;
         md.lcol = d.lcol; md.lval = d.lval; md.seg_begin = d.seg_begin; md.seg_end = d.seg_end;
         md.long_rows = d.long_rows; md.long_segptr = d.long_segptr; md.perm0 = d.perm0; md.iperm0 = d.iperm0;
         md.x_user = r.X; md.y_user = r.Y;

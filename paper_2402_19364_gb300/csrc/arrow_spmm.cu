@@ -49,11 +49,6 @@ void set_error(const std::string& msg) { g_last_error = msg; }
 #ifndef ARROW_ROWS_MIN_BLOCKS_RESCALE
 #define ARROW_ROWS_MIN_BLOCKS_RESCALE 4
 #endif
-// 1: a row's last round has exactly its remaining entries (gather_row); 0: rounds of 8 with
-// the slots past the row's end predicated off (gather_row_pred).
-#ifndef ARROW_ROWS_EXACT
-#define ARROW_ROWS_EXACT 1
-#endif
 // CTAs per SM of the split-row combine kernel's grid (and its launch bound), without and with
 // the FP64 rescale (whose per-lane FP64 sums need more registers).
 #ifndef ARROW_COMB_CTAS_PER_SM
@@ -72,6 +67,7 @@ static inline int rows_smem_bytes(const TileLayout& L, int norm_doubles) { retur
 
 struct RowArgs {
     const int32_t* rowptr;     // short-row stream
+    const uint32_t* row_desc;
     const int32_t* col;
     const void* val;
     const int32_t* tile_row;
@@ -138,7 +134,7 @@ __device__ __forceinline__ void flush_squares(float* sq, double* slot, int lane)
 // Thread 0: stage tile t (row pointers, columns, values) into buf with three bulk copies.
 template <typename TV>
 __device__ __forceinline__ void issue_tile(const RowArgs& a, int t, unsigned char* buf, uint64_t* bar) {
-    stage_tile<TV>(a.rowptr, a.col, static_cast<const TV*>(a.val), a.tile_row[t], a.tile_row[t + 1], a.tile_ent[t],
+    stage_tile<TV>(a.row_desc, a.col, static_cast<const TV*>(a.val), a.tile_row[t], a.tile_row[t + 1], a.tile_ent[t],
                    a.tile_ent[t + 1], buf, bar, a.rp_bytes, a.col_bytes);
 }
 
@@ -206,27 +202,28 @@ __global__ void __launch_bounds__(256, RESCALE ? ARROW_ROWS_MIN_BLOCKS_RESCALE :
             break;
         }
         const int r0 = __ldg(a.tile_row + t), r1 = __ldg(a.tile_row + t + 1), e0 = __ldg(a.tile_ent + t);
-        const int32_t* srp = reinterpret_cast<const int32_t*>(buf) + (r0 & 3);
+        const uint32_t* sdesc = reinterpret_cast<const uint32_t*>(buf) + (r0 & 3);
         const int32_t* scol = reinterpret_cast<const int32_t*>(buf + a.rp_bytes) + (e0 & 3);
         const TV* sval = reinterpret_cast<const TV*>(buf + a.rp_bytes + a.col_bytes) + (e0 & (VE - 1));
         const int nrows = r1 - r0;
-        for (int j = team; j < nrows; j += TEAMS) {
-            const int s = srp[j] - e0, e = srp[j + 1] - e0;
+        // the next row's descriptor is read a row ahead (past the tile's end it is a word of the
+        // same buffer that nothing uses)
+        uint32_t dn = sdesc[team];
+        for (int q = team; q < nrows; q += TEAMS) {
+            const RowDesc rd = row_desc_unpack(dn, a.rowptr, r0);
+            dn = sdesc[q + TEAMS];
+            const int s = rd.start, e = rd.start + rd.len;
             float acc[V];
 #pragma unroll
             for (int v = 0; v < V; ++v) acc[v] = 0.f;
-#if ARROW_ROWS_EXACT
             gather_row<TX, TV>(scol, sval, s, e, X, a.ldx, acc);
-#else
-            gather_row_pred<TX, TV>(scol, sval, s, e, X, a.ldx, acc);
-#endif
             if (RESCALE) {
 #pragma unroll
                 for (int v = 0; v < V; ++v) acc[v] *= scl[v];
             }
             if (a.sigma) apply_sigma<T, V>(acc, a.sigma, lane);
             const uint4 out = P::from_float(acc);
-            st_y(Y + int64_t(r0 + j) * a.ldx, out);
+            st_y(Y + int64_t(r0 + rd.row) * a.ldx, out);
             if (RESCALE) {
                 float yr[V];
                 P::to_float(out, yr);
@@ -276,6 +273,27 @@ __global__ void arrow_selftest_wait_kernel(int32_t* status, uint64_t limit_ns) {
     __syncthreads();
     const bool ok = mbar_wait_bounded(&bar, 0, limit_ns);
     if (__syncthreads_or(!ok) && threadIdx.x == 0) atomicExch(status, kStatusTimeout);
+}
+
+// Row descriptors of every tile (one CTA per tile, row_desc_pack): a row's place is the number of
+// rows of its tile that are longer, or as long and before it.
+__global__ void __launch_bounds__(256) arrow_row_desc_kernel(const int32_t* __restrict__ rowptr,
+                                                             const int32_t* __restrict__ tile_row, int n_tiles,
+                                                             uint32_t* __restrict__ row_desc) {
+    __shared__ int len[kMaxTileRows];
+    for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
+        const int r0 = tile_row[t], nrows = tile_row[t + 1] - r0;
+        const int e0 = rowptr[r0];
+        for (int j = threadIdx.x; j < nrows; j += blockDim.x) len[j] = rowptr[r0 + j + 1] - rowptr[r0 + j];
+        __syncthreads();
+        for (int j = threadIdx.x; j < nrows; j += blockDim.x) {
+            const int l = len[j];
+            int at = 0;
+            for (int i = 0; i < nrows; ++i) at += len[i] > l || (len[i] == l && i < j);
+            row_desc[r0 + at] = row_desc_pack(uint32_t(rowptr[r0 + j] - e0), uint32_t(j), uint32_t(l));
+        }
+        __syncthreads();
+    }
 }
 
 struct SegArgs {
@@ -760,7 +778,7 @@ int cuda_fail(cudaError_t e, const char* what) {
     } while (0)
 
 static void free_device(DeviceData& d) {
-    void* ptrs[] = {d.rowptr, d.col, d.val, d.tile_row, d.tile_ent, d.lcol, d.lval, d.perm0, d.iperm0,
+    void* ptrs[] = {d.rowptr, d.col, d.val, d.tile_row, d.tile_ent, d.row_desc, d.lcol, d.lval, d.perm0, d.iperm0,
                     d.long_rows, d.long_segptr, d.seg_begin, d.seg_end, d.status, d.ws, d.col_v, d.lcol_v};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -855,8 +873,24 @@ static int upload_values(const arrow_handle_s* h, const std::vector<int32_t>& sr
 
 static int upload_to_current(arrow_handle_s* h);
 
-template <typename T>
-static int upload_vec(T** dst, const std::vector<T>& src, size_t& bytes);
+// Row descriptors of the handle's tiles, built on the device from the uploaded row pointers and tile
+// table (allocated once: their number does not depend on the tiling).
+static int build_row_desc(arrow_handle_s* h) {
+    DeviceData& d = h->dev;
+    const int64_t n_tiles = h->tile_row.empty() ? 0 : int64_t(h->tile_row.size()) - 1;
+    if (h->n == 0 || n_tiles == 0) return ARROW_OK;
+    if (!d.row_desc) {
+        const size_t bytes = size_t(h->n) * sizeof(uint32_t) + kPad;
+        ACK(cudaMalloc(&d.row_desc, bytes));
+        d.bytes += bytes;
+        ACK(cudaMemset(reinterpret_cast<char*>(d.row_desc) + size_t(h->n) * sizeof(uint32_t), 0, kPad));
+    }
+    const int grid = int(std::min<int64_t>(n_tiles, int64_t(d.sm_count) * 16));
+    arrow_row_desc_kernel<<<grid, 256>>>(d.rowptr, d.tile_row, int(n_tiles), d.row_desc);
+    ACK(cudaGetLastError());
+    ACK(cudaDeviceSynchronize());
+    return ARROW_OK;
+}
 
 // The column indices as vertex ids (pi_0^{-1} of the stored positions), for a first
 // iteration that gathers straight from the caller's X.  Uploaded when fold_permute_in is set;
@@ -927,7 +961,7 @@ static int upload_to_current(arrow_handle_s* h) {
     if ((rc = upload_values(h, h->f_src, &d.val, d.bytes))) return rc;
     if ((rc = upload_values(h, h->l_src, &d.lval, d.bytes))) return rc;
     if (h->tune.fold_permute_in && (rc = upload_vertex_cols(h))) return rc;
-    return ARROW_OK;
+    return build_row_desc(h);
 }
 
 // ---- launch plumbing -----------------------------------------------------------------
@@ -1050,7 +1084,7 @@ static void launch_step(const arrow_handle_s* h, const Plan& p, const TX* cur, T
             pf.end(ARROW_K_SEGMENTS, e0);
         }
         const TileLayout L = tile_layout(h->tune.tile_rows, h->tune.tile_nnz);
-        RowArgs ra{d.rowptr, col, d.val, d.tile_row, d.tile_ent, n_tiles, cur, nxt, k, koff, p.kc, scale_in, np,
+        RowArgs ra{d.rowptr, d.row_desc, col, d.val, d.tile_row, d.tile_ent, n_tiles, cur, nxt, k, koff, p.kc, scale_in, np,
                    d.status, L.rp, L.col, L.buf, sigma};
         const int smem = rows_smem_bytes(L, np ? 8 * p.kc : 0);
         cudaEvent_t e0 = pf.begin();
@@ -1560,6 +1594,7 @@ int arrow_set_tuning(arrow_handle h, const arrow_tuning* t) {
             int rc;
             if ((rc = upload_vec(&h->dev.tile_row, h->tile_row, bytes))) return rc;
             if ((rc = upload_vec(&h->dev.tile_ent, h->tile_ent, bytes))) return rc;
+            if ((rc = build_row_desc(h))) return rc;
         }
     }
     if (t->fold_permute_in && h->uploaded) {

@@ -10,6 +10,7 @@ namespace arrow {
 
 struct MatDesc {
     const int32_t* rowptr;
+    const uint32_t* row_desc;
     const int32_t* col;
     const void* val;
     const int32_t* tile_row;
@@ -58,19 +59,11 @@ inline int batch_smem_bytes(const TileLayout& L) { return 128 + kStages * L.buf;
 // Rows of every matrix's tiles (the fused arrow-row kernel of arrow_spmm with a per-tile
 // matrix descriptor and a run-time team width); same tile pipeline without block barriers.
 // Resident CTAs per SM that the register use of the batched rows kernel allows (64 registers).
-// Rows are gathered in predicated rounds of 8 (gather_row_pred): measured on 256
-// random-geometric matrices, 47.8 k matrix-iterations/s at 4 CTAs/SM against 44.6 k at 3
-// (80 registers), and 29.2 k with exact-size remainder rounds, whose divergent branch runs
-// the differently sized rounds of a warp's many narrow teams one after the other.
+// A tile's rows come in order of length (row_desc), so the exact-size remainder rounds of
+// gather_row hardly diverge: 24 random-geometric matrices (FP16, k 8..64) 2277 -> 1988 us per
+// 10-iteration call against rows in position order with predicated rounds of 8.
 #ifndef ARROW_BATCH_MIN_BLOCKS
 #define ARROW_BATCH_MIN_BLOCKS 4
-#endif
-// 1: a team sums two rows at a time (gather_row_pair_pred: 4 slots each per round of 8, which
-// needs 80 registers, i.e. 3 CTAs/SM); 0: one row at a time.  256 random-geometric matrices:
-// 48.5 k matrix-iterations/s with pairs at 3 CTAs/SM, 47.6 k one row at a time at 4 (within run
-// to run spread), 35.1 k with pairs squeezed into 64 registers (spills).
-#ifndef ARROW_BATCH_PAIRS
-#define ARROW_BATCH_PAIRS 0
 #endif
 constexpr int kBatchMinBlocks = ARROW_BATCH_MIN_BLOCKS;
 
@@ -91,7 +84,7 @@ __global__ void __launch_bounds__(256, kBatchMinBlocks) arrow_batch_rows_kernel(
         const int t = int(w - a.base[m]);
         const int r0 = d.tile_row[t], r1 = d.tile_row[t + 1], e0 = d.tile_ent[t], e1 = d.tile_ent[t + 1];
         ps->hdr[b][0] = m; ps->hdr[b][1] = r0; ps->hdr[b][2] = r1; ps->hdr[b][3] = e0;
-        stage_tile<TV>(d.rowptr, d.col, static_cast<const TV*>(d.val), r0, r1, e0, e1, bufs + b * a.buf_bytes, &ps->full[b],
+        stage_tile<TV>(d.row_desc, d.col, static_cast<const TV*>(d.val), r0, r1, e0, e1, bufs + b * a.buf_bytes, &ps->full[b],
                        a.rp_bytes, a.col_bytes);
         ps->issued[b]++;
     };
@@ -126,33 +119,18 @@ __global__ void __launch_bounds__(256, kBatchMinBlocks) arrow_batch_rows_kernel(
         const int par = a.parity ^ d.flip;
         const TX* __restrict__ X = static_cast<const TX*>(par ? d.xb : d.xa) + tl * V;
         TX* __restrict__ Y = static_cast<TX*>(par ? d.xa : d.xb) + tl * V;
-        const int32_t* srp = reinterpret_cast<const int32_t*>(buf) + (r0 & 3);
+        const uint32_t* sdesc = reinterpret_cast<const uint32_t*>(buf) + (r0 & 3);
         const int32_t* scol = reinterpret_cast<const int32_t*>(buf + a.rp_bytes) + (e0 & 3);
         const TV* sval = reinterpret_cast<const TV*>(buf + a.rp_bytes + a.col_bytes) + (e0 & (VE - 1));
         const int nrows = r1 - r0;
-#if ARROW_BATCH_PAIRS
-        // two rows per team at a time (gather_row_pair_pred)
-        for (int j = team; j < nrows; j += 2 * teams) {
-            const int j2 = j + teams;
-            const int s = srp[j] - e0, e = srp[j + 1] - e0;
-            const int s2 = j2 < nrows ? srp[j2] - e0 : 0, e2 = j2 < nrows ? srp[j2 + 1] - e0 : 0;
-            float acc[V], acc2[V];
-#pragma unroll
-            for (int v = 0; v < V; ++v) { acc[v] = 0.f; acc2[v] = 0.f; }
-            gather_row_pair_pred<TX, TV>(scol, sval, s, e, s2, e2, X, ldx, acc, acc2);
-            *reinterpret_cast<uint4*>(Y + int64_t(r0 + j) * ldx) = P::from_float(acc);
-            if (j2 < nrows) *reinterpret_cast<uint4*>(Y + int64_t(r0 + j2) * ldx) = P::from_float(acc2);
-        }
-#else
-        for (int j = team; j < nrows; j += teams) {
-            const int s = srp[j] - e0, e = srp[j + 1] - e0;
+        for (int q = team; q < nrows; q += teams) {
+            const RowDesc rd = row_desc_unpack(sdesc[q], d.rowptr, r0);
             float acc[V];
 #pragma unroll
             for (int v = 0; v < V; ++v) acc[v] = 0.f;
-            gather_row_pred<TX, TV>(scol, sval, s, e, X, ldx, acc);
-            *reinterpret_cast<uint4*>(Y + int64_t(r0 + j) * ldx) = P::from_float(acc);
+            gather_row<TX, TV>(scol, sval, rd.start, rd.start + rd.len, X, ldx, acc);
+            *reinterpret_cast<uint4*>(Y + int64_t(r0 + rd.row) * ldx) = P::from_float(acc);
         }
-#endif
         __syncwarp();
         if (lane == 0)
             release_buffer(ps, b, NW, [&](int bb) {

@@ -316,25 +316,11 @@ __device__ __forceinline__ void gather_round(const int32_t* scol, const TV* sval
     for (int u = 0; u < R; ++u) axpy_vec<TX, TV>(sval[base + u], x[u], acc);
 }
 
-// The same round when the row has only cnt (< R) entries left: the slots past cnt are
-// predicated off.
-template <int R, typename TX, typename TV>
-__device__ __forceinline__ void gather_round_upto(const int32_t* scol, const TV* sval, int base, int cnt, const TX* X,
-                                                  int64_t ldx, float* acc) {
-    uint4 x[R];
-#pragma unroll
-    for (int u = 0; u < R; ++u)
-        if (u < cnt) x[u] = ld_x(X + int64_t(scol[base + u]) * ldx);
-#pragma unroll
-    for (int u = 0; u < R; ++u)
-        if (u < cnt) axpy_vec<TX, TV>(sval[base + u], x[u], acc);
-}
-
 // All entries [s, e) of a staged row in entry order: full rounds of 8 gathers, then one round
 // of exactly the remaining 1..7.  A round of 8 with the unused slots predicated off would
 // still issue their instructions (a 9-entry row spent 16 slots); the exact round costs a
-// divergent branch when the teams of a warp have different remainders, which is cheap when a
-// warp holds few teams (wide rows) and costly when it holds many (see gather_row_pred).
+// divergent branch when the teams of a warp have different remainders, which the order of a
+// tile's rows keeps rare (row_desc_pack).
 template <typename TX, typename TV, bool COHERENT = false>
 __device__ __forceinline__ void gather_row(const int32_t* scol, const TV* sval, int s, int e, const TX* X, int64_t ldx,
                                            float* acc) {
@@ -352,36 +338,25 @@ __device__ __forceinline__ void gather_row(const int32_t* scol, const TV* sval, 
     }
 }
 
-// The same sum in rounds of 8 whose slots past the row's end are predicated off: one code
-// path for all the teams of a warp, whatever their row lengths.
-template <typename TX, typename TV>
-__device__ __forceinline__ void gather_row_pred(const int32_t* scol, const TV* sval, int s, int e, const TX* X,
-                                                int64_t ldx, float* acc) {
-    for (int base = s; base < e; base += 8) gather_round_upto<8>(scol, sval, base, e - base, X, ldx, acc);
+// Row descriptors: one 32-bit word per row, every tile's rows in order of decreasing length
+// (equal lengths in row order), so that the teams of a warp walk rows of the same length
+// together.  In row order the exact remainder rounds of gather_row diverge on every warp whose
+// rows differ: a random-geometric warp of 8 teams ran up to 7 remainder sizes one after the
+// other, each with its own memory latency (random-geometric graph, 1 M rows, k = 32 FP16: 96
+// -> 63 us per product; R-MAT 20, k = 128 BF16: 1.09x on the whole call; grids, whose rows are
+// all alike, 0.5-0.8 % slower by the unpacking).  Fields: first entry within the tile (15 bits: a
+// tile has at most 16384 entries), row within the tile (11 bits: at most 2048 rows), length (6
+// bits; kLongDesc means "kLongDesc or more", read from the row pointers).  They take the place of
+// the row pointers in the staged tile: the same bytes.
+constexpr uint32_t kLongDesc = 63;
+__host__ __device__ inline uint32_t row_desc_pack(uint32_t start, uint32_t row, uint32_t len) {
+    return start | (row << 15) | ((len < kLongDesc ? len : kLongDesc) << 26);
 }
-
-// Two rows of a staged tile summed together: rounds of 8 gathers, the first 4 slots for row A
-// and the last 4 for row B (slots past a row's end predicated off), each row accumulated in its
-// own entry order.  A 9-entry row alone takes 2 rounds of 8 slots; two of them together take 3.
-template <typename TX, typename TV>
-__device__ __forceinline__ void gather_row_pair_pred(const int32_t* scol, const TV* sval, int sa, int ea, int sb,
-                                                     int eb, const TX* X, int64_t ldx, float* acca, float* accb) {
-    for (int a = sa, b = sb; a < ea || b < eb; a += 4, b += 4) {
-        const int ca = ea - a, cb = eb - b;
-        uint4 xa[4], xb[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (u < ca) xa[u] = ld_x(X + int64_t(scol[a + u]) * ldx);
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (u < cb) xb[u] = ld_x(X + int64_t(scol[b + u]) * ldx);
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (u < ca) axpy_vec<TX, TV>(sval[a + u], xa[u], acca);
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (u < cb) axpy_vec<TX, TV>(sval[b + u], xb[u], accb);
-    }
+struct RowDesc { int start, row, len; };
+__device__ __forceinline__ RowDesc row_desc_unpack(uint32_t d, const int32_t* __restrict__ rowptr, int r0) {
+    RowDesc r{int(d & 0x7fffu), int((d >> 15) & 0x7ffu), int(d >> 26)};
+    if (r.len == int(kLongDesc)) r.len = __ldg(rowptr + r0 + r.row + 1) - __ldg(rowptr + r0 + r.row);
+    return r;
 }
 
 // Tile pipeline state at the start of dynamic shared memory (128 bytes): one "full"
@@ -434,10 +409,10 @@ __host__ __device__ inline TileLayout tile_layout(int tile_rows, int tile_nnz) {
     return L;
 }
 
-// Stage the row tile [r0, r1) with entries [e0, e1) into buf: row pointers, columns and values,
+// Stage the row tile [r0, r1) with entries [e0, e1) into buf: row descriptors, columns and values,
 // each as a 16-byte aligned superset (the arrays are padded by 64 bytes), completing on bar.
 template <typename TV>
-__device__ __forceinline__ void stage_tile(const int32_t* rowptr, const int32_t* col, const TV* val, int r0, int r1,
+__device__ __forceinline__ void stage_tile(const uint32_t* row_desc, const int32_t* col, const TV* val, int r0, int r1,
                                            int e0, int e1, unsigned char* buf, uint64_t* bar, int rp_bytes,
                                            int col_bytes) {
     constexpr int VE = 16 / int(sizeof(TV));
@@ -448,7 +423,7 @@ __device__ __forceinline__ void stage_tile(const int32_t* rowptr, const int32_t*
     const uint32_t bcol = uint32_t(cb - ca) * 4u;
     const uint32_t bval = uint32_t(vb - va) * uint32_t(sizeof(TV));
     mbar_arrive_expect_tx(bar, brp + bcol + bval);
-    bulk_g2s(buf, rowptr + ra, brp, bar);
+    bulk_g2s(buf, row_desc + ra, brp, bar);
     if (bcol) bulk_g2s(buf + rp_bytes, col + ca, bcol, bar);
     if (bval) bulk_g2s(buf + rp_bytes + col_bytes, val + va, bval, bar);
 }

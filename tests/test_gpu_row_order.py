@@ -1,0 +1,52 @@
+"""GPU test of the length-ordered rows of a tile (row descriptors) at the sizes where their fields end.
+
+Rows of 0 to 140 entries, unsplit (long_row 256): below, at and above the length the descriptor
+holds itself (63), one tile of 2048 rows, tiles of 32 rows, and a last tile of one row.  Tolerances:
+FP32 1e-5 per column against the FP64 oracle (a sum of at most 140 products with relative error
+2^-24 each stays below 140 * 2^-24 = 8.4e-6 of the sum of magnitudes, and the values are positive).
+"""
+import numpy as np
+import pytest
+
+import workloads as w
+from oracle import spmm as S
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def arrow():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2402_19364_gb300 import build
+    build.build()
+    import paper_2402_19364_gb300 as pkg
+    return pkg
+
+
+def _matrix(n):
+    rng = np.random.default_rng(11)
+    special = np.array([0, 1, 7, 8, 9, 15, 16, 17, 61, 62, 63, 64, 65, 127, 128, 140])
+    counts = np.where(rng.random(n) < 0.5, special[rng.integers(0, special.size, n)], rng.integers(0, 20, n))
+    rowptr = np.zeros(n + 1, dtype=np.int64)
+    np.cumsum(counts, out=rowptr[1:])
+    cols = [np.sort(rng.choice(n, c, replace=False)) for c in counts]
+    colidx = np.concatenate(cols).astype(np.int32)
+    vals = rng.uniform(0.5, 1.5, colidx.size).astype(np.float32).astype(np.float64)
+    return w.Csr(n, rowptr, colidx, vals)
+
+
+@pytest.mark.parametrize("tile", [(2048, 8192), (32, 1024), (256, 2048)])
+@pytest.mark.parametrize("k", [4, 16, 128])
+def test_rows_by_length(arrow, tile, k):
+    A = _matrix(2049)
+    M = arrow.ArrowMatrix(A, 64, long_row=256)
+    M.set_tuning(tile[0], tile[1], 2, 70)
+    X = np.abs(w.features(A.n, k, seed=3))
+    Xd = torch.from_numpy(X).cuda()
+    R = S.iterate(A, X.astype(np.float64), 1)
+    for got in (M.spmm(Xd, 1), arrow.ArrowBatch([M]).spmm([Xd], 1)[0]):
+        Y = got.cpu().numpy().astype(np.float64)
+        assert np.all(np.abs(Y - R) <= 1e-5 * np.max(R, axis=0))
