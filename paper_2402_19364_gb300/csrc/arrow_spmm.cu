@@ -512,30 +512,50 @@ __global__ void __launch_bounds__(256) arrow_gather_rows_kernel(const TX* __rest
 // ------------------------------------------------------------------------------------
 // one-launch path for small problems
 // ------------------------------------------------------------------------------------
-// Grid-wide barrier of a cooperative launch (every CTA resident): sense by generation count.
-// Thread 0 of each CTA arrives; the last one resets the counter and advances the generation;
-// the others wait for the generation to move, at most limit_ns.  Returns false (in every
-// thread of the CTA) when the wait ran out.
-__device__ __forceinline__ bool grid_barrier(unsigned* count, unsigned* gen, unsigned G, uint64_t limit_ns) {
+// Grid-wide barrier of a cooperative launch (every CTA resident).  The arrival count only grows:
+// barrier number i of the launch (i = 1, 2, ...) is passed when it reaches i * G, so an arrival is one
+// release add and a wait is acquire loads, with nothing to reset in between.  Thread 0 of each
+// CTA arrives and waits, at most limit_ns; the clock is read once in 64 polls (read on every
+// poll, it made up most of a barrier).  Returns false (in every thread of the CTA) when the wait
+// ran out.
+__device__ __forceinline__ bool grid_barrier(unsigned* count, unsigned target, uint64_t limit_ns) {
     __syncthreads();
     int ok = 1;
     if (threadIdx.x == 0) {
-        volatile unsigned* vg = gen;
-        const unsigned g0 = *vg;
-        __threadfence();
-        if (atomicAdd(count, 1u) == G - 1) {
-            *reinterpret_cast<volatile unsigned*>(count) = 0;
-            __threadfence();
-            atomicAdd(gen, 1u);
-        } else {
-            const uint64_t t0 = global_ns();
-            while (*vg == g0) {
-                if (global_ns() - t0 > limit_ns) { ok = 0; break; }
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
+        uint64_t t0 = 0;
+        for (unsigned polls = 1;; ++polls) {
+            unsigned v;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(count) : "memory");
+            if (int(v - target) >= 0) break;
+            if ((polls & 63) == 0) {
+                const uint64_t now = global_ns();
+                if (t0 == 0) t0 = now;
+                else if (now - t0 > limit_ns) { ok = 0; break; }
             }
         }
-        __threadfence();
     }
     return __syncthreads_and(ok) != 0;
+}
+
+// Sum over the threads' values v of each column c = threadIdx.x % C (C columns, a power of two up to
+// 256): inside a warp by a fixed xor butterfly over the lanes of a column, then the warps in
+// order.  Returns the column's sum in the first C threads.  sh: 8 * C doubles.  Few FP64 adds in a
+// chain: this GPU starts about two FP64 operations per clock and SM, and a serial sum over a
+// CTA's teams (128 adds at k = 8) took longer than the product it followed.
+__device__ __forceinline__ double column_sum(double v, int C, double* sh) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int off = C; off < 32; off <<= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    if (C >= 32) sh[threadIdx.x] = v;                   // thread t: column t % C, group t / C
+    else if (lane < C) sh[warp * C + lane] = v;
+    __syncthreads();
+    double acc = 0.0;
+    if (int(threadIdx.x) < C) {
+        const int groups = C >= 32 ? 256 / C : 8;
+        for (int g = 0; g < groups; ++g) acc += sh[g * C + threadIdx.x];
+    }
+    __syncthreads();
+    return acc;
 }
 
 struct FusedArgs {
@@ -559,7 +579,7 @@ struct FusedArgs {
     double* np;             // [2][gridDim.x][k] FP64 column sums, by iteration parity
     int64_t k;
     int32_t iters, sigma;
-    unsigned* bar;          // [0] arrival count, [1] generation
+    unsigned* bar;          // arrival count, 0 at the start of the launch
     int32_t* status;
 };
 
@@ -570,8 +590,12 @@ struct FusedArgs {
 // computed with the same code and order as the multi-launch path (identical bits without the
 // rescale; with it the column sums are grouped by this launch's CTAs).  Needs k / V <= 32 (one
 // chunk).  A barrier that runs out sets the status word and the kernel returns.
+// Bound by latency: per iteration one row per team (dependent loads of its entries and X rows from
+// L2), a grid barrier, and with the rescale two short FP64 sums.  5,063 rows, k = 8 FP32, 20
+// iterations with the rescale: 211 us per call with serial FP64 sums and a clock read on every
+// poll of the barrier, 108 us in this form.
 template <typename TX, typename TV, int T, bool RESCALE>
-__global__ void __launch_bounds__(256) arrow_fused_small_kernel(FusedArgs a) {
+__global__ void __launch_bounds__(256, 1) arrow_fused_small_kernel(FusedArgs a) {
     using P = Pack<TX>;
     constexpr int V = P::V;
     constexpr int TEAMS = 256 / T;
@@ -583,8 +607,11 @@ __global__ void __launch_bounds__(256) arrow_fused_small_kernel(FusedArgs a) {
     const int64_t gteam = int64_t(blockIdx.x) * TEAMS + team, nteams = G * TEAMS;
     const int64_t gwarp = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5, nwarps = (G * blockDim.x) >> 5;
     const int64_t k = a.k;
-    __shared__ double wsum[TEAMS * T * V];   // per-team FP64 column sums (RESCALE)
-    __shared__ float scl_s[T * V];           // this iteration's column factors
+    constexpr int C = T * V;                 // columns: k
+    __shared__ float wsq[RESCALE ? TEAMS * C : 1];    // the lanes' squares, team by team
+    __shared__ double sh[RESCALE ? 8 * C : 1];
+    __shared__ float scl_s[C];               // this iteration's column factors
+    unsigned passed = 0;                     // barriers so far
     const TV* val = static_cast<const TV*>(a.val);
     const TV* lval = static_cast<const TV*>(a.lval);
 
@@ -596,7 +623,7 @@ __global__ void __launch_bounds__(256) arrow_fused_small_kernel(FusedArgs a) {
             *reinterpret_cast<uint4*>(dst + p * k + col0) = ld_x_cg(src + int64_t(__ldg(a.iperm0 + p)) * k + col0);
     }
     for (int c = threadIdx.x; c < T * V; c += blockDim.x) scl_s[c] = 1.0f;
-    if (!grid_barrier(a.bar, a.bar + 1, unsigned(G), kWaitLimitNs)) {
+    if (!grid_barrier(a.bar, ++passed * unsigned(G), kWaitLimitNs)) {
         if (threadIdx.x == 0) atomicExch(a.status, kStatusTimeout);
         return;
     }
@@ -646,7 +673,7 @@ __global__ void __launch_bounds__(256) arrow_fused_small_kernel(FusedArgs a) {
             }
         }
         if (a.n_long) {
-            if (!grid_barrier(a.bar, a.bar + 1, unsigned(G), kWaitLimitNs)) {
+            if (!grid_barrier(a.bar, ++passed * unsigned(G), kWaitLimitNs)) {
                 if (threadIdx.x == 0) atomicExch(a.status, kStatusTimeout);
                 return;
             }
@@ -682,29 +709,26 @@ __global__ void __launch_bounds__(256) arrow_fused_small_kernel(FusedArgs a) {
             }
         }
         if (RESCALE) {
-            // this CTA's FP64 column sums: lanes' FP32 squares per team, teams in order
+            // this CTA's FP64 column sums: a thread adds every 256 / C-th team's squares of its column
 #pragma unroll
-            for (int v = 0; v < V; ++v) wsum[team * (T * V) + col0 + v] = double(sq[v]);
+            for (int v = 0; v < V; ++v) wsq[team * C + col0 + v] = sq[v];
             __syncthreads();
-            double* npo = a.np + int64_t(t & 1) * G * k;
-            for (int c = threadIdx.x; c < T * V; c += blockDim.x) {
-                double acc = 0.0;
-                for (int t2 = 0; t2 < TEAMS; ++t2) acc += wsum[t2 * (T * V) + c];
-                npo[int64_t(blockIdx.x) * k + c] = acc;
-            }
+            double part = 0.0;
+            for (int e = threadIdx.x; e < TEAMS * C; e += 256) part += double(wsq[e]);
+            const double acc = column_sum(part, C, sh);
+            if (int(threadIdx.x) < C) a.np[(int64_t(t & 1) * G + blockIdx.x) * k + threadIdx.x] = acc;
         }
-        if (!grid_barrier(a.bar, a.bar + 1, unsigned(G), kWaitLimitNs)) {
+        if (!grid_barrier(a.bar, ++passed * unsigned(G), kWaitLimitNs)) {
             if (threadIdx.x == 0) atomicExch(a.status, kStatusTimeout);
             return;
         }
         if (RESCALE) {
             // every CTA sums the partials of all CTAs in the same order: the same factors
             const double* npi = a.np + int64_t(t & 1) * G * k;
-            for (int c = threadIdx.x; c < T * V; c += blockDim.x) {
-                double acc = 0.0;
-                for (int64_t b = 0; b < G; ++b) acc += __ldcg(npi + b * k + c);
-                scl_s[c] = acc > 0.0 ? float(1.0 / sqrt(acc)) : 1.0f;
-            }
+            double part = 0.0;
+            for (int e = threadIdx.x; e < int(G) * C; e += 256) part += __ldcg(npi + e);
+            const double acc = column_sum(part, C, sh);
+            if (int(threadIdx.x) < C) scl_s[threadIdx.x] = acc > 0.0 ? float(1.0 / sqrt(acc)) : 1.0f;
             __syncthreads();
         }
         TX* tmp = cur;
@@ -735,7 +759,7 @@ __global__ void __launch_bounds__(256) arrow_fused_small_kernel(FusedArgs a) {
 // wait must give up after limit_ns; each block that gave up adds 1 to status[0].
 __global__ void arrow_selftest_grid_kernel(unsigned* bar, int32_t* status, uint64_t limit_ns) {
     if (blockIdx.x == 0) return;
-    if (!grid_barrier(bar, bar + 1, gridDim.x, limit_ns) && threadIdx.x == 0) atomicAdd(status, 1);
+    if (!grid_barrier(bar, gridDim.x, limit_ns) && threadIdx.x == 0) atomicAdd(status, 1);
 }
 
 template <typename TV>
