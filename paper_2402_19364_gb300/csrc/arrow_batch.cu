@@ -28,10 +28,11 @@ struct arrow_batch_s {
     int device = -1;
     int value_dtype = ARROW_F32;
     int sm_count = 1;
-    // prefix sums of work units per kernel class: tiles, segments, long rows, 32-row chunks
-    std::vector<int64_t> base[4];
+    // prefix sums of work units per kernel class: tiles, segments, long rows, 32-row chunks, 32-row chunks
+    // of the matrices that keep a permute-out pass (folds_out; by the last call's k and dtype)
+    std::vector<int64_t> base[5];
     std::vector<uint64_t> gens;           // each handle's generation when base/descriptors were built
-    int64_t* d_base = nullptr;            // the four prefix arrays, concatenated
+    int64_t* d_base = nullptr;            // the five prefix arrays, concatenated
     MatDesc* d_desc = nullptr;
     std::vector<MatDesc> h_desc;
     void* ws = nullptr;
@@ -58,8 +59,8 @@ template <typename TX, typename TV>
 void enqueue_typed(arrow_batch_s* B, int iters, cudaStream_t s) {
     const int64_t n_m = int64_t(B->hs.size());
     const int64_t* db = B->d_base;
-    const int64_t tot[4] = {B->base[0].back(), B->base[1].back(), B->base[2].back(), B->base[3].back()};
-    const int64_t* bases[4] = {db, db + (n_m + 1), db + 2 * (n_m + 1), db + 3 * (n_m + 1)};
+    const int64_t tot[5] = {B->base[0].back(), B->base[1].back(), B->base[2].back(), B->base[3].back(), B->base[4].back()};
+    const int64_t* bases[5] = {db, db + (n_m + 1), db + 2 * (n_m + 1), db + 3 * (n_m + 1), db + 4 * (n_m + 1)};
     const int sm = B->sm_count;
     int rows_max = 32, nnz_max = kMinTileNnz, ctas = 3, carve = 75;
     for (const arrow_handle_s* h : B->hs) {
@@ -68,8 +69,8 @@ void enqueue_typed(arrow_batch_s* B, int iters, cudaStream_t s) {
     }
     if (!B->hs.empty()) { ctas = std::min(B->hs[0]->tune.ctas_per_sm, kBatchMinBlocks); carve = B->hs[0]->tune.carveout; }
     const TileLayout L = tile_layout(rows_max, nnz_max);
-    auto args = [&](int cls, int parity, int dir) {
-        return BatchArgs{B->d_desc, bases[cls], int32_t(n_m), tot[cls], parity, dir, B->d_status, L.rp, L.col, L.buf};
+    auto args = [&](int cls, int parity, int dir, int out = 0) {
+        return BatchArgs{B->d_desc, bases[cls], int32_t(n_m), tot[cls], parity, dir, out, B->d_status, L.rp, L.col, L.buf};
     };
     auto grid_w = [&](int64_t units, int per_sm) {   // warp-per-unit kernels
         return int(std::max<int64_t>(1, std::min<int64_t>((units + 7) / 8, int64_t(sm) * per_sm)));
@@ -81,11 +82,11 @@ void enqueue_typed(arrow_batch_s* B, int iters, cudaStream_t s) {
         const int rgrid = int(std::max<int64_t>(1, std::min<int64_t>(tot[0], int64_t(sm) * ctas)));
         if (tot[0]) {
             prepare_batch_rows<TX, TV>(carve);
-            arrow_batch_rows_kernel<TX, TV><<<rgrid, 256, batch_smem_bytes(L), s>>>(args(0, parity, 0));
+            arrow_batch_rows_kernel<TX, TV><<<rgrid, 256, batch_smem_bytes(L), s>>>(args(0, parity, 0, t == iters));
         }
-        if (tot[2]) arrow_batch_combine_kernel<TX><<<grid_w(tot[2], 4), 256, 0, s>>>(args(2, parity, 0));
+        if (tot[2]) arrow_batch_combine_kernel<TX><<<grid_w(tot[2], 4), 256, 0, s>>>(args(2, parity, 0, t == iters));
     }
-    arrow_batch_gather_kernel<TX><<<grid_w(tot[3], 8), 256, 0, s>>>(args(3, iters & 1, 1));
+    if (tot[4]) arrow_batch_gather_kernel<TX><<<grid_w(tot[4], 8), 256, 0, s>>>(args(4, iters & 1, 1));
 }
 
 template <typename TX>
@@ -117,6 +118,7 @@ cudaError_t upload_bases(arrow_batch_s* B) {
         B->base[1].push_back(B->base[1].back() + int64_t(h->seg_begin.size()));
         B->base[2].push_back(B->base[2].back() + int64_t(h->long_rows.size()));
         B->base[3].push_back(B->base[3].back() + (h->n + 31) / 32);
+        B->base[4].push_back(0);
     }
     std::vector<int64_t> all;
     for (auto& v : B->base) all.insert(all.end(), v.begin(), v.end());
@@ -153,7 +155,7 @@ int arrow_batch_create(const arrow_handle* handles, int32_t count, arrow_batch* 
         }
         B->hs.push_back(h);
     }
-    cudaError_t e = cudaMalloc(&B->d_base, 4 * (B->hs.size() + 1) * sizeof(int64_t));
+    cudaError_t e = cudaMalloc(&B->d_base, 5 * (B->hs.size() + 1) * sizeof(int64_t));
     if (e == cudaSuccess) e = upload_bases(B);
     if (e == cudaSuccess) e = cudaMalloc(&B->d_desc, B->hs.size() * sizeof(MatDesc));
     if (e == cudaSuccess) e = cudaMalloc(&B->d_status, sizeof(int32_t));
@@ -254,6 +256,9 @@ int arrow_batch_spmm(arrow_batch B, const void* const* X, void* const* Y, const 
             B->h_desc[m] = md;
         }
         BCK(cudaMemcpy(B->d_desc, B->h_desc.data(), n_m * sizeof(MatDesc), cudaMemcpyHostToDevice));
+        for (size_t m = 0; m < n_m; ++m)
+            B->base[4][m + 1] = B->base[4][m] + (folds_out(k[m], int(dsize(x_dtype))) ? 0 : (B->hs[m]->n + 31) / 32);
+        BCK(cudaMemcpy(B->d_base + 4 * (n_m + 1), B->base[4].data(), (n_m + 1) * sizeof(int64_t), cudaMemcpyHostToDevice));
         B->key = key;
     }
     if (!(flags & ARROW_GRAPH)) {

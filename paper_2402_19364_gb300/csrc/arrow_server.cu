@@ -111,7 +111,7 @@ void launch_step(arrow_server_s* S, const int64_t* tot, int n_m, cudaStream_t s)
     const int ctas = S->active.empty() ? 3 : std::min(S->active[0].h->tune.ctas_per_sm, kBatchMinBlocks);
     const int carve = S->active.empty() ? 75 : S->active[0].h->tune.carveout;
     auto args = [&](int cls, int parity, int dir) {
-        return BatchArgs{S->d_desc, db + cls * (n_m + 1), n_m, tot[cls], parity, dir, S->d_status, L.rp, L.col, L.buf};
+        return BatchArgs{S->d_desc, db + cls * (n_m + 1), n_m, tot[cls], parity, dir, 0, S->d_status, L.rp, L.col, L.buf};
     };
     const int sm = S->sm_count;
     auto grid_w = [&](int64_t units, int per_sm) {
@@ -342,13 +342,14 @@ static int server_step(arrow_server_s* S, void* stream, int32_t* active_out) {
         const bool iterate = r.left > 0;
         const bool finish = r.left <= 1;
         md.flip = iterate ? r.parity : 1;   // a request with no iteration leaves its result in xa
+        md.out = iterate && finish;
         desc[m] = md;
         const int64_t units[kClasses] = {
             r.fresh ? (h->n + 31) / 32 : 0,
             iterate ? int64_t(h->seg_begin.size()) : 0,
             iterate ? (h->tile_row.empty() ? 0 : int64_t(h->tile_row.size()) - 1) : 0,
             iterate ? int64_t(h->long_rows.size()) : 0,
-            finish ? (h->n + 31) / 32 : 0};
+            finish && !(iterate && folds_out(r.k, int(xsize(dt)))) ? (h->n + 31) / 32 : 0};
         for (int c = 0; c < kClasses; ++c) {
             tot[c] += units[c];
             base[c * (n_m + 1) + m + 1] = tot[c];

@@ -81,6 +81,7 @@ struct RowArgs {
     const double* scale;       // [k] per-column factor d_{t-1}, or null
     double* norm_partials;     // [gridDim.x][k] (rows kernel slots), or null
     int32_t* status;
+    const int32_t* out_idx;    // row r is stored at row out_idx[r] of Y (permute-out folded in), or null
     int32_t rp_bytes, col_bytes, buf_bytes;   // shared-memory layout of a staged tile
     int32_t sigma;             // kSigmaRelu | kSigmaRowNorm applied to each output row, or 0
 };
@@ -213,6 +214,7 @@ __global__ void __launch_bounds__(256, RESCALE ? ARROW_ROWS_MIN_BLOCKS_RESCALE :
             const RowDesc rd = row_desc_unpack(dn, a.rowptr, r0);
             dn = sdesc[q + TEAMS];
             const int s = rd.start, e = rd.start + rd.len;
+            const int64_t yr0 = a.out_idx ? __ldg(a.out_idx + r0 + rd.row) : r0 + rd.row;
             float acc[V];
 #pragma unroll
             for (int v = 0; v < V; ++v) acc[v] = 0.f;
@@ -223,7 +225,7 @@ __global__ void __launch_bounds__(256, RESCALE ? ARROW_ROWS_MIN_BLOCKS_RESCALE :
             }
             if (a.sigma) apply_sigma<T, V>(acc, a.sigma, lane);
             const uint4 out = P::from_float(acc);
-            st_y(Y + int64_t(r0 + rd.row) * a.ldx, out);
+            st_y(Y + yr0 * a.ldx, out);
             if (RESCALE) {
                 float yr[V];
                 P::to_float(out, yr);
@@ -348,6 +350,7 @@ struct CombArgs {
     int32_t koff, kc;
     const double* scale;
     double* norm_partials;     // [gridDim.x][k] (combine slots), or null
+    const int32_t* out_idx;    // as RowArgs
     int32_t sigma;
 };
 
@@ -406,7 +409,8 @@ __global__ void __launch_bounds__(256, RESCALE ? ARROW_COMB_CTAS_PER_SM_RESCALE 
         }
         if (a.sigma) apply_sigma<T, V>(acc, a.sigma, lane);
         const uint4 out = P::from_float(acc);
-        *reinterpret_cast<uint4*>(Y + int64_t(__ldg(a.long_rows + li)) * a.ldx) = out;
+        const int32_t r = __ldg(a.long_rows + li);
+        *reinterpret_cast<uint4*>(Y + int64_t(a.out_idx ? __ldg(a.out_idx + r) : r) * a.ldx) = out;
         if (RESCALE) {
             float yr[V];
             P::to_float(out, yr);
@@ -636,6 +640,11 @@ __global__ void __launch_bounds__(256, 1) arrow_fused_small_kernel(FusedArgs a) 
         float sq[V];
 #pragma unroll
         for (int v = 0; v < V; ++v) sq[v] = 0.f;
+        // without the rescale the last iteration stores its rows at their vertices in Y (every CTA has read
+        // the caller's X by then)
+        const bool last = !RESCALE && t == a.iters;
+        TX* dst = last ? static_cast<TX*>(a.Y) : nxt;
+        const int32_t* oidx = last ? a.iperm0 : nullptr;
         // split-row segments (first stage of the head-row reduction)
         for (int64_t g = gwarp; g < a.n_seg; g += nwarps) {
             const int32_t s = __ldg(a.seg_begin + g), e = __ldg(a.seg_end + g);
@@ -664,7 +673,7 @@ __global__ void __launch_bounds__(256, 1) arrow_fused_small_kernel(FusedArgs a) 
             }
             if (a.sigma) apply_sigma<T, V>(acc, a.sigma, lane);
             const uint4 out = P::from_float(acc);
-            *reinterpret_cast<uint4*>(nxt + p * k + col0) = out;
+            *reinterpret_cast<uint4*>(dst + (oidx ? int64_t(__ldg(oidx + p)) : p) * k + col0) = out;
             if (RESCALE && (a.n_long == 0 || s < e)) {   // split rows are summed after the combine
                 float yr[V];
                 P::to_float(out, yr);
@@ -699,7 +708,8 @@ __global__ void __launch_bounds__(256, 1) arrow_fused_small_kernel(FusedArgs a) 
                 }
                 if (a.sigma) apply_sigma<T, V>(acc, a.sigma, lane);
                 const uint4 out = P::from_float(acc);
-                *reinterpret_cast<uint4*>(nxt + int64_t(__ldg(a.long_rows + li)) * k + col0) = out;
+                const int32_t r = __ldg(a.long_rows + li);
+                *reinterpret_cast<uint4*>(dst + int64_t(oidx ? __ldg(oidx + r) : r) * k + col0) = out;
                 if (RESCALE) {
                     float yr[V];
                     P::to_float(out, yr);
@@ -718,6 +728,7 @@ __global__ void __launch_bounds__(256, 1) arrow_fused_small_kernel(FusedArgs a) 
             const double acc = column_sum(part, C, sh);
             if (int(threadIdx.x) < C) a.np[(int64_t(t & 1) * G + blockIdx.x) * k + threadIdx.x] = acc;
         }
+        if (last) return;
         if (!grid_barrier(a.bar, ++passed * unsigned(G), kWaitLimitNs)) {
             if (threadIdx.x == 0) atomicExch(a.status, kStatusTimeout);
             return;
@@ -735,22 +746,18 @@ __global__ void __launch_bounds__(256, 1) arrow_fused_small_kernel(FusedArgs a) 
         cur = nxt;
         nxt = tmp;
     }
-    // permute-out: Y[v] = cur[pi_0(v)] (* the last column factors)
-    {
+    // permute-out with the last column factors: Y[v] = cur[pi_0(v)] * d
+    if (RESCALE) {
         float scl[V];
 #pragma unroll
         for (int v = 0; v < V; ++v) scl[v] = scl_s[col0 + v];
         TX* dst = static_cast<TX*>(a.Y);
         for (int64_t v = gteam; v < a.n; v += nteams) {
-            uint4 o = ld_x_cg(cur + int64_t(__ldg(a.perm0 + v)) * k + col0);
-            if (RESCALE) {
-                float f[V];
-                P::to_float(o, f);
+            float f[V];
+            P::to_float(ld_x_cg(cur + int64_t(__ldg(a.perm0 + v)) * k + col0), f);
 #pragma unroll
-                for (int u = 0; u < V; ++u) f[u] *= scl[u];
-                o = P::from_float(f);
-            }
-            *reinterpret_cast<uint4*>(dst + v * k + col0) = o;
+            for (int u = 0; u < V; ++u) f[u] *= scl[u];
+            *reinterpret_cast<uint4*>(dst + v * k + col0) = P::from_float(f);
         }
     }
 }
@@ -1094,7 +1101,7 @@ static int sigma_of(int flags) {
 template <typename TX, typename TV, int T>
 static void launch_step(const arrow_handle_s* h, const Plan& p, const TX* cur, TX* nxt, int64_t k, float* part,
                         const double* scale_in, double* np, int sigma, const int32_t* col, const int32_t* lcol,
-                        cudaStream_t s, Prof& pf) {
+                        const int32_t* out_idx, cudaStream_t s, Prof& pf) {
     const DeviceData& d = h->dev;
     const int32_t n_tiles = h->tile_row.empty() ? 0 : int32_t(h->tile_row.size()) - 1;
     for (int ch = 0; ch < p.chunks; ++ch) {
@@ -1109,7 +1116,7 @@ static void launch_step(const arrow_handle_s* h, const Plan& p, const TX* cur, T
         }
         const TileLayout L = tile_layout(h->tune.tile_rows, h->tune.tile_nnz);
         RowArgs ra{d.rowptr, d.row_desc, col, d.val, d.tile_row, d.tile_ent, n_tiles, cur, nxt, k, koff, p.kc, scale_in, np,
-                   d.status, L.rp, L.col, L.buf, sigma};
+                   d.status, out_idx, L.rp, L.col, L.buf, sigma};
         const int smem = rows_smem_bytes(L, np ? 8 * p.kc : 0);
         cudaEvent_t e0 = pf.begin();
         if (np) {
@@ -1122,7 +1129,7 @@ static void launch_step(const arrow_handle_s* h, const Plan& p, const TX* cur, T
         pf.end(ARROW_K_ROWS, e0);
         if (p.comb_grid) {
             CombArgs ca{d.long_rows, d.long_segptr, int32_t(h->long_rows.size()), part, nxt, k, koff, p.kc, scale_in,
-                        np ? np + size_t(p.rows_grid) * size_t(k) : nullptr, sigma};
+                        np ? np + size_t(p.rows_grid) * size_t(k) : nullptr, out_idx, sigma};
             cudaEvent_t e1 = pf.begin();
             if (np)
                 arrow_combine_kernel<TX, T, true><<<p.comb_grid, 256, 0, s>>>(ca);
@@ -1133,13 +1140,14 @@ static void launch_step(const arrow_handle_s* h, const Plan& p, const TX* cur, T
     }
 }
 
-// The iterations: step t reads `cur` and writes the other workspace buffer.  The first step
+// The iterations: step t reads `cur` and writes the other workspace buffer, or, the last one with the
+// permute-out folded in (y_out not null), the caller's Y.  The first step
 // reads x_first: the pi_0-ordered copy xa, or (permute-in folded) the caller's X through the
 // vertex-id column indices.
 template <typename TX, typename TV>
 static void run_steps(const arrow_handle_s* h, const Plan& p, const TX* x_first, bool folded, TX* xa, TX* xb,
-                      int64_t k, int iters, int flags, float* part, double* np, double* sc, cudaStream_t s,
-                      TX** final_buf, Prof& pf) {
+                      int64_t k, int iters, int flags, float* part, double* np, double* sc, TX* y_out,
+                      cudaStream_t s, TX** final_buf, Prof& pf) {
     const DeviceData& d = h->dev;
     const TX* cur = x_first;
     TX* nxt = xb;
@@ -1150,13 +1158,15 @@ static void run_steps(const arrow_handle_s* h, const Plan& p, const TX* x_first,
         double* npo = rescale ? np : nullptr;
         const int32_t* col = (folded && t == 1) ? d.col_v : d.col;
         const int32_t* lcol = (folded && t == 1) ? d.lcol_v : d.lcol;
+        const int32_t* oidx = (y_out && t == iters) ? d.iperm0 : nullptr;
+        if (oidx) nxt = y_out;
         switch (p.T) {
-            case 1: launch_step<TX, TV, 1>(h, p, cur, nxt, k, part, sin, npo, sg, col, lcol, s, pf); break;
-            case 2: launch_step<TX, TV, 2>(h, p, cur, nxt, k, part, sin, npo, sg, col, lcol, s, pf); break;
-            case 4: launch_step<TX, TV, 4>(h, p, cur, nxt, k, part, sin, npo, sg, col, lcol, s, pf); break;
-            case 8: launch_step<TX, TV, 8>(h, p, cur, nxt, k, part, sin, npo, sg, col, lcol, s, pf); break;
-            case 16: launch_step<TX, TV, 16>(h, p, cur, nxt, k, part, sin, npo, sg, col, lcol, s, pf); break;
-            default: launch_step<TX, TV, 32>(h, p, cur, nxt, k, part, sin, npo, sg, col, lcol, s, pf); break;
+            case 1: launch_step<TX, TV, 1>(h, p, cur, nxt, k, part, sin, npo, sg, col, lcol, oidx, s, pf); break;
+            case 2: launch_step<TX, TV, 2>(h, p, cur, nxt, k, part, sin, npo, sg, col, lcol, oidx, s, pf); break;
+            case 4: launch_step<TX, TV, 4>(h, p, cur, nxt, k, part, sin, npo, sg, col, lcol, oidx, s, pf); break;
+            case 8: launch_step<TX, TV, 8>(h, p, cur, nxt, k, part, sin, npo, sg, col, lcol, oidx, s, pf); break;
+            case 16: launch_step<TX, TV, 16>(h, p, cur, nxt, k, part, sin, npo, sg, col, lcol, oidx, s, pf); break;
+            default: launch_step<TX, TV, 32>(h, p, cur, nxt, k, part, sin, npo, sg, col, lcol, oidx, s, pf); break;
         }
         if (rescale) {
             cudaEvent_t e0 = pf.begin();
@@ -1213,6 +1223,19 @@ static int launch_fused(const arrow_handle_s* h, const Plan& p, const void* X, i
     return ARROW_OK;
 }
 
+// Whether the last iteration stores its rows straight into the caller's Y (row p at vertex
+// pi_0^{-1}(p)) instead of a permute-out reading and writing them once more.  Not with the column
+// rescale, whose last factors are known only after the last row.  Not for rows of less than a
+// 32-byte sector, which scattered stores would write in halves.  And not when the same launch
+// reads the caller's X (one iteration with the permute-in folded in) and X and Y overlap.
+static bool fold_permute_out(const arrow_handle_s* h, const void* X, const void* Y, int64_t k, int sx, int iters, int flags,
+                             bool folded_in) {
+    const size_t bytes = size_t(h->n) * size_t(k) * size_t(sx);
+    if ((flags & ARROW_RESCALE) || k * sx < 32) return false;
+    const uintptr_t x = reinterpret_cast<uintptr_t>(X), y = reinterpret_cast<uintptr_t>(Y);
+    return !(folded_in && iters == 1 && x < y + bytes && y < x + bytes);
+}
+
 template <typename TX>
 static int spmm_typed(const arrow_handle_s* h, const Plan& p, const void* X, int64_t k, int iters, void* Y, int flags,
                       char* ws, cudaStream_t s, Prof& pf) {
@@ -1236,15 +1259,18 @@ static int spmm_typed(const arrow_handle_s* h, const Plan& p, const void* X, int
     }
     const TX* first = folded ? static_cast<const TX*>(X) : xa;
     TX* fin = xa;
+    TX* y_out = fold_permute_out(h, X, Y, k, int(sizeof(TX)), iters, flags, folded) ? static_cast<TX*>(Y) : nullptr;
     switch (h->opts.value_dtype) {
-        case ARROW_F32: run_steps<TX, float>(h, p, first, folded, xa, xb, k, iters, flags, part, np, sc, s, &fin, pf); break;
-        case ARROW_BF16: run_steps<TX, __nv_bfloat16>(h, p, first, folded, xa, xb, k, iters, flags, part, np, sc, s, &fin, pf); break;
-        default: run_steps<TX, __half>(h, p, first, folded, xa, xb, k, iters, flags, part, np, sc, s, &fin, pf); break;
+        case ARROW_F32: run_steps<TX, float>(h, p, first, folded, xa, xb, k, iters, flags, part, np, sc, y_out, s, &fin, pf); break;
+        case ARROW_BF16: run_steps<TX, __nv_bfloat16>(h, p, first, folded, xa, xb, k, iters, flags, part, np, sc, y_out, s, &fin, pf); break;
+        default: run_steps<TX, __half>(h, p, first, folded, xa, xb, k, iters, flags, part, np, sc, y_out, s, &fin, pf); break;
     }
-    const double* final_scale = (flags & ARROW_RESCALE) ? sc + (iters & 1) * k : nullptr;
-    e0 = pf.begin();
-    arrow_gather_rows_kernel<TX><<<ggrid, 256, 0, s>>>(fin, static_cast<TX*>(Y), d.perm0, n, k, final_scale);
-    pf.end(ARROW_K_PERMUTE, e0);
+    if (!y_out) {
+        const double* final_scale = (flags & ARROW_RESCALE) ? sc + (iters & 1) * k : nullptr;
+        e0 = pf.begin();
+        arrow_gather_rows_kernel<TX><<<ggrid, 256, 0, s>>>(fin, static_cast<TX*>(Y), d.perm0, n, k, final_scale);
+        pf.end(ARROW_K_PERMUTE, e0);
+    }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "arrow_spmm: kernel launch");
     return ARROW_OK;

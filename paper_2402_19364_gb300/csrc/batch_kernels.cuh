@@ -32,6 +32,8 @@ struct MatDesc {
     int64_t k;
     int32_t T;            // lanes per row = k / V
     int32_t flip;         // xor-ed into the launch parity (per-request ping-pong state)
+    int32_t out;          // 1: this launch's iteration is the last, its rows go to y_user
+    int32_t pad;
 };
 
 struct BatchArgs {
@@ -41,6 +43,7 @@ struct BatchArgs {
     int64_t total;
     int32_t parity;        // 0: xa -> xb, 1: xb -> xa
     int32_t dir;           // gather: 0 permute-in, 1 permute-out
+    int32_t out;           // rows, combine: the last iteration of every matrix (MatDesc::out)
     int32_t* status;
     int32_t rp_bytes, col_bytes, buf_bytes;   // staged-tile layout (rows kernel)
 };
@@ -53,6 +56,11 @@ __device__ __forceinline__ int find_mat(const int64_t* base, int n, int64_t w) {
     }
     return lo;
 }
+
+// The last iteration of a matrix stores its rows straight at their vertices in the caller's Y
+// (row p at pi_0^{-1}(p)), without a permute-out pass; rows narrower than a 32-byte sector keep
+// the pass, which would be written in halves.
+__host__ __device__ inline bool folds_out(int64_t k, int sx) { return k * sx >= 32; }
 
 inline int batch_smem_bytes(const TileLayout& L) { return 128 + kStages * L.buf; }
 
@@ -118,18 +126,21 @@ __global__ void __launch_bounds__(256, kBatchMinBlocks) arrow_batch_rows_kernel(
         const int64_t ldx = d.k;
         const int par = a.parity ^ d.flip;
         const TX* __restrict__ X = static_cast<const TX*>(par ? d.xb : d.xa) + tl * V;
-        TX* __restrict__ Y = static_cast<TX*>(par ? d.xa : d.xb) + tl * V;
+        const bool fin = (a.out | d.out) && folds_out(ldx, int(sizeof(TX)));
+        const int32_t* oidx = fin ? d.iperm0 + r0 : nullptr;
+        TX* __restrict__ Y = static_cast<TX*>(fin ? d.y_user : par ? d.xa : d.xb) + tl * V;
         const uint32_t* sdesc = reinterpret_cast<const uint32_t*>(buf) + (r0 & 3);
         const int32_t* scol = reinterpret_cast<const int32_t*>(buf + a.rp_bytes) + (e0 & 3);
         const TV* sval = reinterpret_cast<const TV*>(buf + a.rp_bytes + a.col_bytes) + (e0 & (VE - 1));
         const int nrows = r1 - r0;
         for (int q = team; q < nrows; q += teams) {
             const RowDesc rd = row_desc_unpack(sdesc[q], d.rowptr, r0);
+            const int64_t yr = oidx ? __ldg(oidx + rd.row) : r0 + rd.row;
             float acc[V];
 #pragma unroll
             for (int v = 0; v < V; ++v) acc[v] = 0.f;
             gather_row<TX, TV>(scol, sval, rd.start, rd.start + rd.len, X, ldx, acc);
-            *reinterpret_cast<uint4*>(Y + int64_t(r0 + rd.row) * ldx) = P::from_float(acc);
+            *reinterpret_cast<uint4*>(Y + yr * ldx) = P::from_float(acc);
         }
         __syncwarp();
         if (lane == 0)
@@ -217,8 +228,10 @@ __global__ void __launch_bounds__(256) arrow_batch_combine_kernel(BatchArgs a) {
                 acc[4 * q + 0] += f.x; acc[4 * q + 1] += f.y; acc[4 * q + 2] += f.z; acc[4 * q + 3] += f.w;
             }
         }
-        TX* Y = static_cast<TX*>((a.parity ^ d.flip) ? d.xa : d.xb);
-        *reinterpret_cast<uint4*>(Y + int64_t(__ldg(d.long_rows + li)) * d.k + lane * V) = P::from_float(acc);
+        const bool fin = (a.out | d.out) && folds_out(d.k, int(sizeof(TX)));
+        TX* Y = static_cast<TX*>(fin ? d.y_user : (a.parity ^ d.flip) ? d.xa : d.xb);
+        const int32_t r = __ldg(d.long_rows + li);
+        *reinterpret_cast<uint4*>(Y + int64_t(fin ? __ldg(d.iperm0 + r) : r) * d.k + lane * V) = P::from_float(acc);
     }
 }
 
