@@ -75,26 +75,25 @@ void enqueue_typed(arrow_batch_s* B, int iters, cudaStream_t s) {
     auto grid_w = [&](int64_t units, int per_sm) {   // warp-per-unit kernels
         return int(std::max<int64_t>(1, std::min<int64_t>((units + 7) / 8, int64_t(sm) * per_sm)));
     };
-    arrow_batch_gather_kernel<TX><<<grid_w(tot[3], 8), 256, 0, s>>>(args(3, 0, 0));
+    Launcher go{s, carve, true};
+    go(arrow_batch_gather_kernel<TX>, grid_w(tot[3], 8), 256, 0, args(3, 0, 0));
     for (int t = 1; t <= iters; ++t) {
         const int parity = (t - 1) & 1;
-        if (tot[1]) arrow_batch_segments_kernel<TX, TV><<<grid_w(tot[1], 8), 256, 0, s>>>(args(1, parity, 0));
+        if (tot[1]) go(arrow_batch_segments_kernel<TX, TV>, grid_w(tot[1], 8), 256, 0, args(1, parity, 0));
         const int rgrid = int(std::max<int64_t>(1, std::min<int64_t>(tot[0], int64_t(sm) * ctas)));
         if (tot[0]) {
-            prepare_batch_rows<TX, TV>(carve);
-            arrow_batch_rows_kernel<TX, TV><<<rgrid, 256, batch_smem_bytes(L), s>>>(args(0, parity, 0, t == iters));
+            go(arrow_batch_rows_kernel<TX, TV>, rgrid, 256, batch_smem_bytes(L), args(0, parity, 0, t == iters));
         }
-        if (tot[2]) arrow_batch_combine_kernel<TX><<<grid_w(tot[2], 4), 256, 0, s>>>(args(2, parity, 0, t == iters));
+        if (tot[2]) go(arrow_batch_combine_kernel<TX>, grid_w(tot[2], 4), 256, 0, args(2, parity, 0, t == iters));
     }
-    if (tot[4]) arrow_batch_gather_kernel<TX><<<grid_w(tot[4], 8), 256, 0, s>>>(args(4, iters & 1, 1));
+    if (tot[4]) go(arrow_batch_gather_kernel<TX>, grid_w(tot[4], 8), 256, 0, args(4, iters & 1, 1));
 }
 
 template <typename TX>
 void enqueue_x(arrow_batch_s* B, int iters, cudaStream_t s) {
     switch (B->value_dtype) {
         case ARROW_F32: enqueue_typed<TX, float>(B, iters, s); break;
-        case ARROW_BF16: enqueue_typed<TX, __nv_bfloat16>(B, iters, s); break;
-        default: enqueue_typed<TX, __half>(B, iters, s); break;
+        default: enqueue_typed<TX, TX>(B, iters, s); break;   // checked: the features' type
     }
 }
 

@@ -40,10 +40,10 @@ using uvec = std::vector<T, DefaultInitAlloc<T>>;
 // would read memory that GPU does not own.
 int require_device(int device, const char* what);
 
-// Opt a kernel into the large dynamic shared memory and set its shared-memory carveout.
-// Both are attributes of the kernel in the current device's context, so they are cached per
-// (device, kernel) and re-applied when the carveout changes.
-void set_smem_attrs(const void* fn, int carveout);
+// Opt a kernel into the large dynamic shared memory (if `dynamic`) and set its shared-memory
+// carveout.  Both are attributes of the kernel in the current device's context, so they are
+// cached per (device, kernel) and re-applied when the carveout changes.
+void set_smem_attrs(const void* fn, int carveout, bool dynamic);
 
 // Row tiles of the fused row program: by default at most kTileRows rows and kTileNnz entries
 // each (arrow_set_tuning / arrow_autotune change them per handle).  A tile's row pointers and

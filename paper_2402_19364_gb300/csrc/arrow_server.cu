@@ -117,23 +117,22 @@ void launch_step(arrow_server_s* S, const int64_t* tot, int n_m, cudaStream_t s)
     auto grid_w = [&](int64_t units, int per_sm) {
         return int(std::max<int64_t>(1, std::min<int64_t>((units + 7) / 8, int64_t(sm) * per_sm)));
     };
-    if (tot[0]) arrow_batch_gather_kernel<TX><<<grid_w(tot[0], 8), 256, 0, s>>>(args(0, 0, 0));
-    if (tot[1]) arrow_batch_segments_kernel<TX, TV><<<grid_w(tot[1], 8), 256, 0, s>>>(args(1, 0, 0));
+    Launcher go{s, carve, true};
+    if (tot[0]) go(arrow_batch_gather_kernel<TX>, grid_w(tot[0], 8), 256, 0, args(0, 0, 0));
+    if (tot[1]) go(arrow_batch_segments_kernel<TX, TV>, grid_w(tot[1], 8), 256, 0, args(1, 0, 0));
     if (tot[2]) {
-        prepare_batch_rows<TX, TV>(carve);
         const int g = int(std::max<int64_t>(1, std::min<int64_t>(tot[2], int64_t(sm) * ctas)));
-        arrow_batch_rows_kernel<TX, TV><<<g, 256, batch_smem_bytes(L), s>>>(args(2, 0, 0));
+        go(arrow_batch_rows_kernel<TX, TV>, g, 256, batch_smem_bytes(L), args(2, 0, 0));
     }
-    if (tot[3]) arrow_batch_combine_kernel<TX><<<grid_w(tot[3], 4), 256, 0, s>>>(args(3, 0, 0));
-    if (tot[4]) arrow_batch_gather_kernel<TX><<<grid_w(tot[4], 8), 256, 0, s>>>(args(4, 1, 1));
+    if (tot[3]) go(arrow_batch_combine_kernel<TX>, grid_w(tot[3], 4), 256, 0, args(3, 0, 0));
+    if (tot[4]) go(arrow_batch_gather_kernel<TX>, grid_w(tot[4], 8), 256, 0, args(4, 1, 1));
 }
 
 template <typename TX>
 void launch_x(arrow_server_s* S, int vdt, const int64_t* tot, int n_m, cudaStream_t s) {
     switch (vdt) {
         case ARROW_F32: launch_step<TX, float>(S, tot, n_m, s); break;
-        case ARROW_BF16: launch_step<TX, __nv_bfloat16>(S, tot, n_m, s); break;
-        default: launch_step<TX, __half>(S, tot, n_m, s); break;
+        default: launch_step<TX, TX>(S, tot, n_m, s); break;   // checked: the features' type
     }
 }
 

@@ -184,6 +184,7 @@ __global__ void __launch_bounds__(256, RESCALE ? ARROW_ROWS_MIN_BLOCKS_RESCALE :
                 issue_tile<TV>(a, blockIdx.x + b * G, bufs + b * a.buf_bytes, &ps->full[b]);
                 ps->issued[b]++;
             }
+    pdl_wait();
     // the previous step's column factors (only with the rescale: otherwise there are none, and
     // the registers are left to the gathers)
     float scl[V];
@@ -248,6 +249,7 @@ __global__ void __launch_bounds__(256, RESCALE ? ARROW_ROWS_MIN_BLOCKS_RESCALE :
                 }
             });
     }
+    pdl_launch();
     if (RESCALE) flush_squares<T, V>(sq, wsum + (threadIdx.x >> 5) * a.kc + col0, lane);
     __syncthreads();
     if (ps->failed) {
@@ -324,6 +326,7 @@ __global__ void __launch_bounds__(256, ARROW_SEG_MIN_BLOCKS) arrow_segments_kern
     const int64_t nwarps = (int64_t(gridDim.x) * blockDim.x) >> 5;
     const TX* __restrict__ X = static_cast<const TX*>(a.X) + a.koff + col0;
     const TV* __restrict__ val = static_cast<const TV*>(a.val);
+    pdl_wait();
     for (int64_t g = warp0; g < a.n_seg; g += nwarps) {
         const int32_t s = __ldg(a.seg_begin + g), e = __ldg(a.seg_end + g);
         float acc[V];
@@ -367,6 +370,7 @@ __global__ void __launch_bounds__(256, RESCALE ? ARROW_COMB_CTAS_PER_SM_RESCALE 
     const int64_t team0 = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) / T;
     const int64_t nteams = (int64_t(gridDim.x) * blockDim.x) / T;
     TX* __restrict__ Y = static_cast<TX*>(a.Y) + a.koff + col0;
+    pdl_wait();
     float scl[V];
 #pragma unroll
     for (int v = 0; v < V; ++v) scl[v] = (RESCALE && a.scale) ? float(a.scale[a.koff + col0 + v]) : 1.0f;
@@ -442,6 +446,8 @@ __global__ void __launch_bounds__(256) arrow_norm_finalize_kernel(const double* 
                                                                   double* scale_out) {
     const int64_t c = blockIdx.x;
     double t = 0.0;
+    pdl_wait();
+    pdl_launch();
     for (int p = threadIdx.x; p < nparts; p += blockDim.x) t += partials[int64_t(p) * k + c];
     __shared__ double sh[256];
     sh[threadIdx.x] = t;
@@ -457,12 +463,13 @@ __global__ void __launch_bounds__(256) arrow_norm_finalize_kernel(const double* 
 // a power of two <= 32 (a warp covers 32 / nv rows per pass) or a multiple of 32 (a warp per
 // row); every thread keeps U row gathers in flight.
 template <typename TX>
-__global__ void __launch_bounds__(256) arrow_gather_rows_kernel(const TX* __restrict__ src, TX* __restrict__ dst,
+__global__ void __launch_bounds__(256) arrow_gather_rows_kernel(const TX* src, TX* dst,
                                                                 const int32_t* __restrict__ idx, int64_t n, int64_t k,
-                                                                const double* __restrict__ scale) {
+                                                                const double* scale) {
     using P = Pack<TX>;
     constexpr int V = P::V;
     constexpr int U = 8;
+    pdl_wait();
     const int nv = int(k / V);
     const int lane = threadIdx.x & 31;
     const int64_t warp = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
@@ -1006,7 +1013,7 @@ struct Plan {
 
 // Shared-memory opt-in and carveout of a kernel, cached per (device, kernel): both are
 // attributes in the current device's context, so a second GPU needs its own opt-in.
-void set_smem_attrs(const void* fn, int carveout) {
+void set_smem_attrs(const void* fn, int carveout, bool dynamic) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return;   // the launch that follows reports the error
     struct Seen { int dev; const void* fn; int carveout; };
@@ -1021,7 +1028,7 @@ void set_smem_attrs(const void* fn, int carveout) {
             }
             return;
         }
-    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    if (dynamic) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, carveout);
     seen.push_back({dev, fn, carveout});
 }
@@ -1101,7 +1108,7 @@ static int sigma_of(int flags) {
 template <typename TX, typename TV, int T>
 static void launch_step(const arrow_handle_s* h, const Plan& p, const TX* cur, TX* nxt, int64_t k, float* part,
                         const double* scale_in, double* np, int sigma, const int32_t* col, const int32_t* lcol,
-                        const int32_t* out_idx, cudaStream_t s, Prof& pf) {
+                        const int32_t* out_idx, Launcher& go, Prof& pf) {
     const DeviceData& d = h->dev;
     const int32_t n_tiles = h->tile_row.empty() ? 0 : int32_t(h->tile_row.size()) - 1;
     for (int ch = 0; ch < p.chunks; ++ch) {
@@ -1111,7 +1118,7 @@ static void launch_step(const arrow_handle_s* h, const Plan& p, const TX* cur, T
             const int64_t warps = int64_t(h->seg_begin.size());
             const int grid = int(std::max<int64_t>(1, std::min<int64_t>((warps + 7) / 8, int64_t(d.sm_count) * 8)));
             cudaEvent_t e0 = pf.begin();
-            arrow_segments_kernel<TX, TV, T><<<grid, 256, 0, s>>>(sa);
+            go(arrow_segments_kernel<TX, TV, T>, grid, 256, 0, sa);
             pf.end(ARROW_K_SEGMENTS, e0);
         }
         const TileLayout L = tile_layout(h->tune.tile_rows, h->tune.tile_nnz);
@@ -1120,11 +1127,9 @@ static void launch_step(const arrow_handle_s* h, const Plan& p, const TX* cur, T
         const int smem = rows_smem_bytes(L, np ? 8 * p.kc : 0);
         cudaEvent_t e0 = pf.begin();
         if (np) {
-            set_smem_attrs(reinterpret_cast<const void*>(arrow_rows_kernel<TX, TV, T, true>), h->tune.carveout);
-            arrow_rows_kernel<TX, TV, T, true><<<p.rows_grid, 256, smem, s>>>(ra);
+            go(arrow_rows_kernel<TX, TV, T, true>, p.rows_grid, 256, smem, ra);
         } else {
-            set_smem_attrs(reinterpret_cast<const void*>(arrow_rows_kernel<TX, TV, T, false>), h->tune.carveout);
-            arrow_rows_kernel<TX, TV, T, false><<<p.rows_grid, 256, smem, s>>>(ra);
+            go(arrow_rows_kernel<TX, TV, T, false>, p.rows_grid, 256, smem, ra);
         }
         pf.end(ARROW_K_ROWS, e0);
         if (p.comb_grid) {
@@ -1132,9 +1137,9 @@ static void launch_step(const arrow_handle_s* h, const Plan& p, const TX* cur, T
                         np ? np + size_t(p.rows_grid) * size_t(k) : nullptr, out_idx, sigma};
             cudaEvent_t e1 = pf.begin();
             if (np)
-                arrow_combine_kernel<TX, T, true><<<p.comb_grid, 256, 0, s>>>(ca);
+                go(arrow_combine_kernel<TX, T, true>, p.comb_grid, 256, 0, ca);
             else
-                arrow_combine_kernel<TX, T, false><<<p.comb_grid, 256, 0, s>>>(ca);
+                go(arrow_combine_kernel<TX, T, false>, p.comb_grid, 256, 0, ca);
             pf.end(ARROW_K_SEGMENTS, e1);
         }
     }
@@ -1147,7 +1152,7 @@ static void launch_step(const arrow_handle_s* h, const Plan& p, const TX* cur, T
 template <typename TX, typename TV>
 static void run_steps(const arrow_handle_s* h, const Plan& p, const TX* x_first, bool folded, TX* xa, TX* xb,
                       int64_t k, int iters, int flags, float* part, double* np, double* sc, TX* y_out,
-                      cudaStream_t s, TX** final_buf, Prof& pf) {
+                      Launcher& go, TX** final_buf, Prof& pf) {
     const DeviceData& d = h->dev;
     const TX* cur = x_first;
     TX* nxt = xb;
@@ -1161,16 +1166,16 @@ static void run_steps(const arrow_handle_s* h, const Plan& p, const TX* x_first,
         const int32_t* oidx = (y_out && t == iters) ? d.iperm0 : nullptr;
         if (oidx) nxt = y_out;
         switch (p.T) {
-            case 1: launch_step<TX, TV, 1>(h, p, cur, nxt, k, part, sin, npo, sg, col, lcol, oidx, s, pf); break;
-            case 2: launch_step<TX, TV, 2>(h, p, cur, nxt, k, part, sin, npo, sg, col, lcol, oidx, s, pf); break;
-            case 4: launch_step<TX, TV, 4>(h, p, cur, nxt, k, part, sin, npo, sg, col, lcol, oidx, s, pf); break;
-            case 8: launch_step<TX, TV, 8>(h, p, cur, nxt, k, part, sin, npo, sg, col, lcol, oidx, s, pf); break;
-            case 16: launch_step<TX, TV, 16>(h, p, cur, nxt, k, part, sin, npo, sg, col, lcol, oidx, s, pf); break;
-            default: launch_step<TX, TV, 32>(h, p, cur, nxt, k, part, sin, npo, sg, col, lcol, oidx, s, pf); break;
+            case 1: launch_step<TX, TV, 1>(h, p, cur, nxt, k, part, sin, npo, sg, col, lcol, oidx, go, pf); break;
+            case 2: launch_step<TX, TV, 2>(h, p, cur, nxt, k, part, sin, npo, sg, col, lcol, oidx, go, pf); break;
+            case 4: launch_step<TX, TV, 4>(h, p, cur, nxt, k, part, sin, npo, sg, col, lcol, oidx, go, pf); break;
+            case 8: launch_step<TX, TV, 8>(h, p, cur, nxt, k, part, sin, npo, sg, col, lcol, oidx, go, pf); break;
+            case 16: launch_step<TX, TV, 16>(h, p, cur, nxt, k, part, sin, npo, sg, col, lcol, oidx, go, pf); break;
+            default: launch_step<TX, TV, 32>(h, p, cur, nxt, k, part, sin, npo, sg, col, lcol, oidx, go, pf); break;
         }
         if (rescale) {
             cudaEvent_t e0 = pf.begin();
-            arrow_norm_finalize_kernel<<<int(k), 256, 0, s>>>(np, p.rows_grid + p.comb_grid, k, sc + (t & 1) * k);
+            go(arrow_norm_finalize_kernel, int(k), 256, 0, np, p.rows_grid + p.comb_grid, k, sc + (t & 1) * k);
             pf.end(ARROW_K_NORM, e0);
         }
         cur = nxt;
@@ -1215,8 +1220,7 @@ static int launch_fused(const arrow_handle_s* h, const Plan& p, const void* X, i
     const bool rescale = flags & ARROW_RESCALE;
     switch (h->opts.value_dtype) {
         case ARROW_F32: e = launch_fused_v<TX, float>(p, fa, rescale, s); break;
-        case ARROW_BF16: e = launch_fused_v<TX, __nv_bfloat16>(p, fa, rescale, s); break;
-        default: e = launch_fused_v<TX, __half>(p, fa, rescale, s); break;
+        default: e = launch_fused_v<TX, TX>(p, fa, rescale, s); break;   // check_spmm_args: the features' type
     }
     pf.end(ARROW_K_FUSED, e0);
     if (e != cudaSuccess) return cuda_fail(e, "arrow_spmm: one-launch path");
@@ -1251,24 +1255,24 @@ static int spmm_typed(const arrow_handle_s* h, const Plan& p, const void* X, int
     const int ggrid = int(std::max<int64_t>(1, std::min<int64_t>((vecs + 2047) / 2048, int64_t(d.sm_count) * 8)));
     // permute-in, unless the first iteration reads the caller's X through vertex-id indices
     const bool folded = h->tune.fold_permute_in && (d.col_v || d.lcol_v);
+    Launcher go{s, h->tune.carveout, !pf.h};
     cudaEvent_t e0 = nullptr;
     if (!folded) {
         e0 = pf.begin();
-        arrow_gather_rows_kernel<TX><<<ggrid, 256, 0, s>>>(static_cast<const TX*>(X), xa, d.iperm0, n, k, nullptr);
+        go(arrow_gather_rows_kernel<TX>, ggrid, 256, 0, static_cast<const TX*>(X), xa, d.iperm0, n, k, nullptr);
         pf.end(ARROW_K_PERMUTE, e0);
     }
     const TX* first = folded ? static_cast<const TX*>(X) : xa;
     TX* fin = xa;
     TX* y_out = fold_permute_out(h, X, Y, k, int(sizeof(TX)), iters, flags, folded) ? static_cast<TX*>(Y) : nullptr;
     switch (h->opts.value_dtype) {
-        case ARROW_F32: run_steps<TX, float>(h, p, first, folded, xa, xb, k, iters, flags, part, np, sc, y_out, s, &fin, pf); break;
-        case ARROW_BF16: run_steps<TX, __nv_bfloat16>(h, p, first, folded, xa, xb, k, iters, flags, part, np, sc, y_out, s, &fin, pf); break;
-        default: run_steps<TX, __half>(h, p, first, folded, xa, xb, k, iters, flags, part, np, sc, y_out, s, &fin, pf); break;
+        case ARROW_F32: run_steps<TX, float>(h, p, first, folded, xa, xb, k, iters, flags, part, np, sc, y_out, go, &fin, pf); break;
+        default: run_steps<TX, TX>(h, p, first, folded, xa, xb, k, iters, flags, part, np, sc, y_out, go, &fin, pf); break;
     }
     if (!y_out) {
         const double* final_scale = (flags & ARROW_RESCALE) ? sc + (iters & 1) * k : nullptr;
         e0 = pf.begin();
-        arrow_gather_rows_kernel<TX><<<ggrid, 256, 0, s>>>(fin, static_cast<TX*>(Y), d.perm0, n, k, final_scale);
+        go(arrow_gather_rows_kernel<TX>, ggrid, 256, 0, fin, static_cast<TX*>(Y), d.perm0, n, k, final_scale);
         pf.end(ARROW_K_PERMUTE, e0);
     }
     cudaError_t e = cudaGetLastError();

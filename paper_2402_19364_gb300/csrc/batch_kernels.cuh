@@ -109,6 +109,8 @@ __global__ void __launch_bounds__(256, kBatchMinBlocks) arrow_batch_rows_kernel(
     if (threadIdx.x == 0)
         for (int b = 0; b < kStages; ++b)
             if (int64_t(blockIdx.x) + b * G < a.total) issue(blockIdx.x + b * G, b);
+    pdl_wait();
+    pdl_launch();
     int i = 0;
     for (int64_t w = blockIdx.x; w < a.total; w += G, ++i) {
         const int b = i % kStages;
@@ -153,13 +155,6 @@ __global__ void __launch_bounds__(256, kBatchMinBlocks) arrow_batch_rows_kernel(
     if (ps->failed && threadIdx.x == 0) drain_pipeline(ps);
 }
 
-// Opt the batched rows kernel into large dynamic shared memory and set its carveout (cached
-// per device and kernel instantiation).
-template <typename TX, typename TV>
-inline void prepare_batch_rows(int carveout) {
-    set_smem_attrs(reinterpret_cast<const void*>(arrow_batch_rows_kernel<TX, TV>), carveout);
-}
-
 // One warp per split-row segment of any matrix (first stage of the head-row reduction): the
 // same arithmetic as arrow_segments_kernel, dispatched on the matrix's team width.
 template <typename TX, typename TV, int T>
@@ -187,6 +182,7 @@ __global__ void __launch_bounds__(256, ARROW_SEG_MIN_BLOCKS) arrow_batch_segment
     const int lane = threadIdx.x & 31;
     const int64_t warp0 = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = (int64_t(gridDim.x) * blockDim.x) >> 5;
+    pdl_wait();
     for (int64_t w = warp0; w < a.total; w += nwarps) {
         const int m = find_mat(a.base, a.n_mats, w);
         const MatDesc& d = a.d[m];
@@ -211,6 +207,7 @@ __global__ void __launch_bounds__(256) arrow_batch_combine_kernel(BatchArgs a) {
     const int lane = threadIdx.x & 31;
     const int64_t warp0 = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = (int64_t(gridDim.x) * blockDim.x) >> 5;
+    pdl_wait();
     for (int64_t w = warp0; w < a.total; w += nwarps) {
         const int m = find_mat(a.base, a.n_mats, w);
         const MatDesc& d = a.d[m];
@@ -244,6 +241,7 @@ __global__ void __launch_bounds__(256) arrow_batch_gather_kernel(BatchArgs a) {
     const int lane = threadIdx.x & 31;
     const int64_t warp0 = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = (int64_t(gridDim.x) * blockDim.x) >> 5;
+    pdl_wait();
     for (int64_t w = warp0; w < a.total; w += nwarps) {
         const int m = find_mat(a.base, a.n_mats, w);
         const MatDesc& d = a.d[m];
