@@ -69,8 +69,9 @@ void enqueue_typed(arrow_batch_s* B, int iters, cudaStream_t s) {
     }
     if (!B->hs.empty()) { ctas = std::min(B->hs[0]->tune.ctas_per_sm, kBatchMinBlocks); carve = B->hs[0]->tune.carveout; }
     const TileLayout L = tile_layout(rows_max, nnz_max);
+    const int parts = row_parts(tot[0], int64_t(sm) * ctas, rows_max, 32);
     auto args = [&](int cls, int parity, int dir, int out = 0) {
-        return BatchArgs{B->d_desc, bases[cls], int32_t(n_m), tot[cls], parity, dir, out, B->d_status, L.rp, L.col, L.buf};
+        return BatchArgs{B->d_desc, bases[cls], int32_t(n_m), tot[cls], parity, dir, out, B->d_status, L.rp, L.col, L.buf, parts};
     };
     auto grid_w = [&](int64_t units, int per_sm) {   // warp-per-unit kernels
         return int(std::max<int64_t>(1, std::min<int64_t>((units + 7) / 8, int64_t(sm) * per_sm)));
@@ -80,7 +81,7 @@ void enqueue_typed(arrow_batch_s* B, int iters, cudaStream_t s) {
     for (int t = 1; t <= iters; ++t) {
         const int parity = (t - 1) & 1;
         if (tot[1]) go(arrow_batch_segments_kernel<TX, TV>, grid_w(tot[1], 8), 256, 0, args(1, parity, 0));
-        const int rgrid = int(std::max<int64_t>(1, std::min<int64_t>(tot[0], int64_t(sm) * ctas)));
+        const int rgrid = int(std::max<int64_t>(1, std::min<int64_t>(tot[0] * parts, int64_t(sm) * ctas)));
         if (tot[0]) {
             go(arrow_batch_rows_kernel<TX, TV>, rgrid, 256, batch_smem_bytes(L), args(0, parity, 0, t == iters));
         }
@@ -255,9 +256,13 @@ int arrow_batch_spmm(arrow_batch B, const void* const* X, void* const* Y, const 
             B->h_desc[m] = md;
         }
         BCK(cudaMemcpy(B->d_desc, B->h_desc.data(), n_m * sizeof(MatDesc), cudaMemcpyHostToDevice));
+        std::vector<int64_t> pass(n_m + 1, 0);   // changes with k and dtype only, not with X and Y
         for (size_t m = 0; m < n_m; ++m)
-            B->base[4][m + 1] = B->base[4][m] + (folds_out(k[m], int(dsize(x_dtype))) ? 0 : (B->hs[m]->n + 31) / 32);
-        BCK(cudaMemcpy(B->d_base + 4 * (n_m + 1), B->base[4].data(), (n_m + 1) * sizeof(int64_t), cudaMemcpyHostToDevice));
+            pass[m + 1] = pass[m] + (folds_out(k[m], int(dsize(x_dtype))) ? 0 : (B->hs[m]->n + 31) / 32);
+        if (pass != B->base[4]) {
+            BCK(cudaMemcpy(B->d_base + 4 * (n_m + 1), pass.data(), pass.size() * sizeof(int64_t), cudaMemcpyHostToDevice));
+            B->base[4] = pass;
+        }
         B->key = key;
     }
     if (!(flags & ARROW_GRAPH)) {

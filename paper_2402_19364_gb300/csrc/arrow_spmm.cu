@@ -73,6 +73,7 @@ struct RowArgs {
     const int32_t* tile_row;
     const int32_t* tile_ent;
     int32_t n_tiles;
+    int32_t parts;             // CTAs that share a tile's rows (row_parts)
     const void* X;             // pi_0-ordered input, n x ldx
     void* Y;                   // pi_0-ordered output, n x ldx
     int64_t ldx;               // k
@@ -164,7 +165,8 @@ __global__ void __launch_bounds__(256, RESCALE ? ARROW_ROWS_MIN_BLOCKS_RESCALE :
     const int col0 = tl * V;
     const TX* __restrict__ X = static_cast<const TX*>(a.X) + a.koff + col0;
     TX* __restrict__ Y = static_cast<TX*>(a.Y) + a.koff + col0;
-    const int G = gridDim.x;
+    const int G = gridDim.x, U = a.n_tiles * a.parts;   // units: (tile, part of its rows)
+    auto tile_of = [&](int u) { return a.parts == 1 ? u : u / a.parts; };
 
     if (threadIdx.x == 0) {
         for (int b = 0; b < kStages; ++b) {
@@ -180,8 +182,8 @@ __global__ void __launch_bounds__(256, RESCALE ? ARROW_ROWS_MIN_BLOCKS_RESCALE :
     __syncthreads();
     if (threadIdx.x == 0)
         for (int b = 0; b < kStages; ++b)
-            if (int(blockIdx.x) + b * G < a.n_tiles) {
-                issue_tile<TV>(a, blockIdx.x + b * G, bufs + b * a.buf_bytes, &ps->full[b]);
+            if (int(blockIdx.x) + b * G < U) {
+                issue_tile<TV>(a, tile_of(blockIdx.x + b * G), bufs + b * a.buf_bytes, &ps->full[b]);
                 ps->issued[b]++;
             }
     pdl_wait();
@@ -195,7 +197,8 @@ __global__ void __launch_bounds__(256, RESCALE ? ARROW_ROWS_MIN_BLOCKS_RESCALE :
     for (int v = 0; v < V; ++v) sq[v] = 0.f;
 
     int i = 0;
-    for (int t = blockIdx.x; t < a.n_tiles; t += G, ++i) {
+    for (int u = blockIdx.x; u < U; u += G, ++i) {
+        const int t = tile_of(u), q0 = a.parts == 1 ? team : (u - t * a.parts) * TEAMS + team;
         const int b = i % kStages;
         unsigned char* buf = bufs + b * a.buf_bytes;
         const bool ok = mbar_wait_bounded(&ps->full[b], (i / kStages) & 1, kWaitLimitNs);
@@ -208,12 +211,12 @@ __global__ void __launch_bounds__(256, RESCALE ? ARROW_ROWS_MIN_BLOCKS_RESCALE :
         const int32_t* scol = reinterpret_cast<const int32_t*>(buf + a.rp_bytes) + (e0 & 3);
         const TV* sval = reinterpret_cast<const TV*>(buf + a.rp_bytes + a.col_bytes) + (e0 & (VE - 1));
         const int nrows = r1 - r0;
-        // the next row's descriptor is read a row ahead (past the tile's end it is a word of the
-        // same buffer that nothing uses)
-        uint32_t dn = sdesc[team];
-        for (int q = team; q < nrows; q += TEAMS) {
+        // the next row's descriptor is read a row ahead (the word after the last is never used)
+        const int step = TEAMS * a.parts;
+        uint32_t dn = sdesc[min(q0, nrows)];
+        for (int q = q0; q < nrows; q += step) {
             const RowDesc rd = row_desc_unpack(dn, a.rowptr, r0);
-            dn = sdesc[q + TEAMS];
+            dn = sdesc[min(q + step, nrows)];
             const int s = rd.start, e = rd.start + rd.len;
             const int64_t yr0 = a.out_idx ? __ldg(a.out_idx + r0 + rd.row) : r0 + rd.row;
             float acc[V];
@@ -242,9 +245,9 @@ __global__ void __launch_bounds__(256, RESCALE ? ARROW_ROWS_MIN_BLOCKS_RESCALE :
         __syncwarp();
         if (lane == 0)
             release_buffer(ps, b, NW, [&](int bb) {
-                const int tn = t + kStages * G;
-                if (tn < a.n_tiles) {
-                    issue_tile<TV>(a, tn, bufs + bb * a.buf_bytes, &ps->full[bb]);
+                const int un = u + kStages * G;
+                if (un < U) {
+                    issue_tile<TV>(a, tile_of(un), bufs + bb * a.buf_bytes, &ps->full[bb]);
                     ps->issued[bb]++;
                 }
             });
@@ -1006,6 +1009,7 @@ static int upload_to_current(arrow_handle_s* h) {
 struct Plan {
     int V, T, chunks, kc;
     int fused_grid;  // CTAs of the one-launch path (arrow_fused_small_kernel), 0 = multi-launch path
+    int parts;       // CTAs that share a tile's rows (row_parts)
     int rows_grid;   // CTAs of the rows kernel (= its FP64 norm partial slots)
     int comb_grid;   // CTAs of the combine kernel (= its partial slots after the rows kernel's)
     size_t x_bytes, part_bytes, np_bytes, sc_bytes, total;
@@ -1074,7 +1078,9 @@ static int make_plan(const arrow_handle_s* h, int64_t k, int x_dtype, int flags,
     // (one FP64 norm slot each)
     const int64_t n_tiles = h->tile_row.empty() ? 0 : int64_t(h->tile_row.size()) - 1;
     const int cap = (flags & ARROW_RESCALE) ? ARROW_ROWS_MIN_BLOCKS_RESCALE : ARROW_ROWS_MIN_BLOCKS;
-    p.rows_grid = int(std::max<int64_t>(1, std::min<int64_t>(n_tiles, int64_t(sm) * std::min(h->tune.ctas_per_sm, cap))));
+    const int64_t most = int64_t(sm) * std::min(h->tune.ctas_per_sm, cap);
+    p.parts = row_parts(n_tiles, most, h->tune.tile_rows, 256 / p.T);
+    p.rows_grid = int(std::max<int64_t>(1, std::min<int64_t>(n_tiles * p.parts, most)));
     const int64_t n_long = int64_t(h->long_rows.size());
     const int64_t teams = 256 / p.T;
     // combine kernel: as many CTAs per SM as its launch bound allows (each team has only a split
@@ -1122,7 +1128,7 @@ static void launch_step(const arrow_handle_s* h, const Plan& p, const TX* cur, T
             pf.end(ARROW_K_SEGMENTS, e0);
         }
         const TileLayout L = tile_layout(h->tune.tile_rows, h->tune.tile_nnz);
-        RowArgs ra{d.rowptr, d.row_desc, col, d.val, d.tile_row, d.tile_ent, n_tiles, cur, nxt, k, koff, p.kc, scale_in, np,
+        RowArgs ra{d.rowptr, d.row_desc, col, d.val, d.tile_row, d.tile_ent, n_tiles, p.parts, cur, nxt, k, koff, p.kc, scale_in, np,
                    d.status, out_idx, L.rp, L.col, L.buf, sigma};
         const int smem = rows_smem_bytes(L, np ? 8 * p.kc : 0);
         cudaEvent_t e0 = pf.begin();

@@ -46,6 +46,7 @@ struct BatchArgs {
     int32_t out;           // rows, combine: the last iteration of every matrix (MatDesc::out)
     int32_t* status;
     int32_t rp_bytes, col_bytes, buf_bytes;   // staged-tile layout (rows kernel)
+    int32_t parts;         // rows kernel: CTAs that share a tile's rows (row_parts); unit w is tile w / parts
 };
 
 __device__ __forceinline__ int find_mat(const int64_t* base, int n, int64_t w) {
@@ -86,7 +87,9 @@ __global__ void __launch_bounds__(256, kBatchMinBlocks) arrow_batch_rows_kernel(
     unsigned char* bufs = smem + 128;
     const int lane = threadIdx.x & 31;
     const int64_t G = gridDim.x;
-    auto issue = [&](int64_t w, int b) {
+    const int64_t U = a.total * a.parts;
+    auto issue = [&](int64_t u, int b) {
+        const int64_t w = a.parts == 1 ? u : int64_t(uint32_t(u) / uint32_t(a.parts));   // parts > 1: U < 2^31
         const int m = find_mat(a.base, a.n_mats, w);
         const MatDesc& d = a.d[m];
         const int t = int(w - a.base[m]);
@@ -108,11 +111,11 @@ __global__ void __launch_bounds__(256, kBatchMinBlocks) arrow_batch_rows_kernel(
     __syncthreads();
     if (threadIdx.x == 0)
         for (int b = 0; b < kStages; ++b)
-            if (int64_t(blockIdx.x) + b * G < a.total) issue(blockIdx.x + b * G, b);
+            if (int64_t(blockIdx.x) + b * G < U) issue(blockIdx.x + b * G, b);
     pdl_wait();
     pdl_launch();
     int i = 0;
-    for (int64_t w = blockIdx.x; w < a.total; w += G, ++i) {
+    for (int64_t w = blockIdx.x; w < U; w += G, ++i) {
         const int b = i % kStages;
         unsigned char* buf = bufs + b * a.buf_bytes;
         const bool ok = mbar_wait_bounded(&ps->full[b], (i / kStages) & 1, kWaitLimitNs);
@@ -135,7 +138,8 @@ __global__ void __launch_bounds__(256, kBatchMinBlocks) arrow_batch_rows_kernel(
         const int32_t* scol = reinterpret_cast<const int32_t*>(buf + a.rp_bytes) + (e0 & 3);
         const TV* sval = reinterpret_cast<const TV*>(buf + a.rp_bytes + a.col_bytes) + (e0 & (VE - 1));
         const int nrows = r1 - r0;
-        for (int q = team; q < nrows; q += teams) {
+        const int part = a.parts == 1 ? 0 : int(uint32_t(w) % uint32_t(a.parts));
+        for (int q = team + part * teams; q < nrows; q += teams * a.parts) {
             const RowDesc rd = row_desc_unpack(sdesc[q], d.rowptr, r0);
             const int64_t yr = oidx ? __ldg(oidx + rd.row) : r0 + rd.row;
             float acc[V];
@@ -148,7 +152,7 @@ __global__ void __launch_bounds__(256, kBatchMinBlocks) arrow_batch_rows_kernel(
         if (lane == 0)
             release_buffer(ps, b, NW, [&](int bb) {
                 const int64_t wn = w + kStages * G;
-                if (wn < a.total) issue(wn, bb);
+                if (wn < U) issue(wn, bb);
             });
     }
     __syncthreads();

@@ -7,6 +7,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <utility>
 
@@ -452,6 +453,16 @@ __host__ __device__ inline TileLayout tile_layout(int tile_rows, int tile_nnz) {
     L.col = ((tile_nnz + 8) * 4 + 15) / 16 * 16;
     L.buf = (L.rp + 2 * L.col + 127) / 128 * 128;   // values take at most as much as columns
     return L;
+}
+
+// CTAs that share the rows of one tile.  Fewer tiles than resident CTAs (`most`) leave SMs idle while
+// every team walks several rows, each a chain of dependent loads: then as many CTAs as there is
+// room for stage the same tile, and each takes every parts-th group of rows, down to one row per
+// team.  64 x 64 grid (16 tiles, 4 rows per team), 10 iterations: 44.5 -> 36 us per call.
+inline int row_parts(int64_t n_tiles, int64_t most, int tile_rows, int teams) {
+    if (n_tiles <= 0) return 1;
+    const int64_t useful = (tile_rows + teams - 1) / teams;
+    return int(std::max<int64_t>(1, std::min<int64_t>(useful, most / n_tiles)));
 }
 
 // Stage the row tile [r0, r1) with entries [e0, e1) into buf: row descriptors, columns and values,
