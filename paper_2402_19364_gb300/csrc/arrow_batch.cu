@@ -80,7 +80,9 @@ void enqueue_typed(arrow_batch_s* B, int iters, cudaStream_t s) {
     go(arrow_batch_gather_kernel<TX>, grid_w(tot[3], 8), 256, 0, args(3, 0, 0));
     for (int t = 1; t <= iters; ++t) {
         const int parity = (t - 1) & 1;
-        if (tot[1]) go(arrow_batch_segments_kernel<TX, TV>, grid_w(tot[1], 8), 256, 0, args(1, parity, 0));
+        if (tot[1])
+            go(seg_ahead(tot[1], sm) ? arrow_batch_segments_kernel<TX, TV, true> : arrow_batch_segments_kernel<TX, TV, false>,
+               grid_w(tot[1], 8), 256, 0, args(1, parity, 0));
         const int rgrid = int(std::max<int64_t>(1, std::min<int64_t>(tot[0] * parts, int64_t(sm) * ctas)));
         if (tot[0]) {
             go(arrow_batch_rows_kernel<TX, TV>, rgrid, 256, batch_smem_bytes(L), args(0, parity, 0, t == iters));

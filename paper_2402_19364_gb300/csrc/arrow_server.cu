@@ -120,7 +120,9 @@ void launch_step(arrow_server_s* S, const int64_t* tot, int n_m, cudaStream_t s)
     };
     Launcher go{s, carve, true};
     if (tot[0]) go(arrow_batch_gather_kernel<TX>, grid_w(tot[0], 8), 256, 0, args(0, 0, 0));
-    if (tot[1]) go(arrow_batch_segments_kernel<TX, TV>, grid_w(tot[1], 8), 256, 0, args(1, 0, 0));
+    if (tot[1])
+        go(seg_ahead(tot[1], sm) ? arrow_batch_segments_kernel<TX, TV, true> : arrow_batch_segments_kernel<TX, TV, false>,
+           grid_w(tot[1], 8), 256, 0, args(1, 0, 0));
     if (tot[2]) {
         const int g = int(std::max<int64_t>(1, std::min<int64_t>(tot[2] * parts, int64_t(sm) * ctas)));
         go(arrow_batch_rows_kernel<TX, TV>, g, 256, batch_smem_bytes(L), args(2, 0, 0));

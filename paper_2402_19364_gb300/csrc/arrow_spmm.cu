@@ -316,9 +316,9 @@ struct SegArgs {
 };
 
 // One warp per segment of a split row (segment_partial), teams combined with a fixed xor
-// butterfly (first stage of the deterministic head-row reduction).
-template <typename TX, typename TV, int T>
-__global__ void __launch_bounds__(256, ARROW_SEG_MIN_BLOCKS) arrow_segments_kernel(SegArgs a) {
+// butterfly (first stage of the deterministic head-row reduction).  AHEAD: segment_partial_ahead.
+template <typename TX, typename TV, int T, bool AHEAD>
+__global__ void __launch_bounds__(256, AHEAD ? 1 : ARROW_SEG_MIN_BLOCKS) arrow_segments_kernel(SegArgs a) {
     using P = Pack<TX>;
     constexpr int V = P::V;
     const int lane = threadIdx.x & 31;
@@ -333,7 +333,8 @@ __global__ void __launch_bounds__(256, ARROW_SEG_MIN_BLOCKS) arrow_segments_kern
     for (int64_t g = warp0; g < a.n_seg; g += nwarps) {
         const int32_t s = __ldg(a.seg_begin + g), e = __ldg(a.seg_end + g);
         float acc[V];
-        segment_partial<TX, TV, T>(a.col, val, X, a.ldx, s, e, lane, acc);
+        if constexpr (AHEAD) segment_partial_ahead<TX, TV, T>(a.col, val, X, a.ldx, s, e, lane, acc);
+        else segment_partial<TX, TV, T>(a.col, val, X, a.ldx, s, e, lane, acc);
 #pragma unroll
         for (int off = T; off < 32; off <<= 1)
 #pragma unroll
@@ -659,7 +660,7 @@ __global__ void __launch_bounds__(256, 1) arrow_fused_small_kernel(FusedArgs a) 
         for (int64_t g = gwarp; g < a.n_seg; g += nwarps) {
             const int32_t s = __ldg(a.seg_begin + g), e = __ldg(a.seg_end + g);
             float acc[V];
-            segment_partial<TX, TV, T, 8, true>(a.lcol, lval, cur + col0, k, s, e, lane, acc);
+            segment_partial_ahead<TX, TV, T, true>(a.lcol, lval, cur + col0, k, s, e, lane, acc);
 #pragma unroll
             for (int off = T; off < 32; off <<= 1)
 #pragma unroll
@@ -1124,7 +1125,8 @@ static void launch_step(const arrow_handle_s* h, const Plan& p, const TX* cur, T
             const int64_t warps = int64_t(h->seg_begin.size());
             const int grid = int(std::max<int64_t>(1, std::min<int64_t>((warps + 7) / 8, int64_t(d.sm_count) * 8)));
             cudaEvent_t e0 = pf.begin();
-            go(arrow_segments_kernel<TX, TV, T>, grid, 256, 0, sa);
+            if (seg_ahead(warps, d.sm_count)) go(arrow_segments_kernel<TX, TV, T, true>, grid, 256, 0, sa);
+            else go(arrow_segments_kernel<TX, TV, T, false>, grid, 256, 0, sa);
             pf.end(ARROW_K_SEGMENTS, e0);
         }
         const TileLayout L = tile_layout(h->tune.tile_rows, h->tune.tile_nnz);

@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(256, kBatchMinBlocks) arrow_batch_rows_kernel(
 
 // One warp per split-row segment of any matrix (first stage of the head-row reduction): the
 // same arithmetic as arrow_segments_kernel, dispatched on the matrix's team width.
-template <typename TX, typename TV, int T>
+template <typename TX, typename TV, int T, bool AHEAD>
 __device__ __forceinline__ void batch_segment(const MatDesc& d, int64_t g, int par, int lane) {
     using P = Pack<TX>;
     constexpr int V = P::V;
@@ -169,7 +169,8 @@ __device__ __forceinline__ void batch_segment(const MatDesc& d, int64_t g, int p
     const TX* __restrict__ X = static_cast<const TX*>(par ? d.xb : d.xa) + tl * V;
     const int32_t s = __ldg(d.seg_begin + g), e = __ldg(d.seg_end + g);
     float acc[V];
-    segment_partial<TX, TV, T>(d.lcol, static_cast<const TV*>(d.lval), X, d.k, s, e, lane, acc);
+    if constexpr (AHEAD) segment_partial_ahead<TX, TV, T>(d.lcol, static_cast<const TV*>(d.lval), X, d.k, s, e, lane, acc);
+    else segment_partial<TX, TV, T>(d.lcol, static_cast<const TV*>(d.lval), X, d.k, s, e, lane, acc);
 #pragma unroll
     for (int off = T; off < 32; off <<= 1)
 #pragma unroll
@@ -181,8 +182,8 @@ __device__ __forceinline__ void batch_segment(const MatDesc& d, int64_t g, int p
     }
 }
 
-template <typename TX, typename TV>
-__global__ void __launch_bounds__(256, ARROW_SEG_MIN_BLOCKS) arrow_batch_segments_kernel(BatchArgs a) {
+template <typename TX, typename TV, bool AHEAD>
+__global__ void __launch_bounds__(256, AHEAD ? 1 : ARROW_SEG_MIN_BLOCKS) arrow_batch_segments_kernel(BatchArgs a) {
     const int lane = threadIdx.x & 31;
     const int64_t warp0 = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = (int64_t(gridDim.x) * blockDim.x) >> 5;
@@ -193,12 +194,12 @@ __global__ void __launch_bounds__(256, ARROW_SEG_MIN_BLOCKS) arrow_batch_segment
         const int64_t g = w - a.base[m];
         const int par = a.parity ^ d.flip;
         switch (d.T) {
-            case 1: batch_segment<TX, TV, 1>(d, g, par, lane); break;
-            case 2: batch_segment<TX, TV, 2>(d, g, par, lane); break;
-            case 4: batch_segment<TX, TV, 4>(d, g, par, lane); break;
-            case 8: batch_segment<TX, TV, 8>(d, g, par, lane); break;
-            case 16: batch_segment<TX, TV, 16>(d, g, par, lane); break;
-            default: batch_segment<TX, TV, 32>(d, g, par, lane); break;
+            case 1: batch_segment<TX, TV, 1, AHEAD>(d, g, par, lane); break;
+            case 2: batch_segment<TX, TV, 2, AHEAD>(d, g, par, lane); break;
+            case 4: batch_segment<TX, TV, 4, AHEAD>(d, g, par, lane); break;
+            case 8: batch_segment<TX, TV, 8, AHEAD>(d, g, par, lane); break;
+            case 16: batch_segment<TX, TV, 16, AHEAD>(d, g, par, lane); break;
+            default: batch_segment<TX, TV, 32, AHEAD>(d, g, par, lane); break;
         }
     }
 }

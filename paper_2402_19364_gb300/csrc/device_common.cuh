@@ -284,10 +284,6 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
 #ifndef ARROW_SEG_MIN_BLOCKS
 #define ARROW_SEG_MIN_BLOCKS 4
 #endif
-// 1: a segment's last 1..7 entries of a team are gathered in one round; 0: one at a time.
-#ifndef ARROW_SEG_EXACT_TAIL
-#define ARROW_SEG_EXACT_TAIL 1
-#endif
 // R entries j, j + S, ..., j + (R-1) S of a split-row segment (columns and values from
 // global memory), their gathers issued together, accumulated in that order.
 template <int R, typename TX, typename TV, int S, bool COHERENT = false>
@@ -304,6 +300,23 @@ __device__ __forceinline__ void segment_tail(const int32_t* __restrict__ col, co
     for (int u = 0; u < R; ++u) x[u] = ld_row<COHERENT>(X + int64_t(c[u]) * ldx);
 #pragma unroll
     for (int u = 0; u < R; ++u) axpy_vec<TX, TV>(w[u], x[u], acc);
+}
+
+// The team's last 0..7 entries j, j + TPW, ...: one round of exactly that many gathers (one at a
+// time, each would wait a full latency); same order of accumulation.
+template <typename TX, typename TV, int TPW, bool COHERENT>
+__device__ __forceinline__ void segment_rest(const int32_t* __restrict__ col, const TV* __restrict__ val,
+                                             const TX* __restrict__ X, int64_t ldx, int j, int e, float* acc) {
+    switch (j < e ? (e - j + TPW - 1) / TPW : 0) {
+        case 7: segment_tail<7, TX, TV, TPW, COHERENT>(col, val, X, ldx, j, acc); break;
+        case 6: segment_tail<6, TX, TV, TPW, COHERENT>(col, val, X, ldx, j, acc); break;
+        case 5: segment_tail<5, TX, TV, TPW, COHERENT>(col, val, X, ldx, j, acc); break;
+        case 4: segment_tail<4, TX, TV, TPW, COHERENT>(col, val, X, ldx, j, acc); break;
+        case 3: segment_tail<3, TX, TV, TPW, COHERENT>(col, val, X, ldx, j, acc); break;
+        case 2: segment_tail<2, TX, TV, TPW, COHERENT>(col, val, X, ldx, j, acc); break;
+        case 1: segment_tail<1, TX, TV, TPW, COHERENT>(col, val, X, ldx, j, acc); break;
+        default: break;
+    }
 }
 
 template <typename TX, typename TV, int T, int U = 8, bool COHERENT = false>
@@ -331,23 +344,58 @@ __device__ __forceinline__ void segment_partial(const int32_t* __restrict__ col,
 #pragma unroll
         for (int u = 0; u < U; ++u) axpy_vec<TX, TV>(w[u], x[u], acc);
     }
-#if ARROW_SEG_EXACT_TAIL
-    // the team's last 0..U-1 entries j, j + TPW, ...: one round of exactly that many gathers
-    // (one at a time, each would wait a full latency); same order of accumulation
-    switch (j < e ? (e - j + TPW - 1) / TPW : 0) {
-        case 7: segment_tail<7, TX, TV, TPW, COHERENT>(col, val, X, ldx, j, acc); break;
-        case 6: segment_tail<6, TX, TV, TPW, COHERENT>(col, val, X, ldx, j, acc); break;
-        case 5: segment_tail<5, TX, TV, TPW, COHERENT>(col, val, X, ldx, j, acc); break;
-        case 4: segment_tail<4, TX, TV, TPW, COHERENT>(col, val, X, ldx, j, acc); break;
-        case 3: segment_tail<3, TX, TV, TPW, COHERENT>(col, val, X, ldx, j, acc); break;
-        case 2: segment_tail<2, TX, TV, TPW, COHERENT>(col, val, X, ldx, j, acc); break;
-        case 1: segment_tail<1, TX, TV, TPW, COHERENT>(col, val, X, ldx, j, acc); break;
-        default: break;
-    }
-#else
-    for (; j < e; j += TPW) segment_tail<1, TX, TV, TPW, COHERENT>(col, val, X, ldx, j, acc);
-#endif
+    segment_rest<TX, TV, TPW, COHERENT>(col, val, X, ldx, j, e, acc);
 }
+
+// segment_partial where a launch has few segments: the same entries in the same order (the same bits),
+// 16 gathers in flight instead of 8 and the next 16 columns and values loaded while they fly, so a
+// long segment is a chain of a quarter as many memory latencies.  It takes about 150 registers (8
+// warps per SM), so it is used where those warps take at most one segment each (seg_ahead): R-MAT
+// 13, 892 segments, 10 iterations 290 -> 260 us per call at k = 128 BF16 and 162 -> 150 at k = 16
+// FP32, 299 -> 268 on the one-launch path (which has one CTA per SM and always takes it); with
+// 2,374 segments it lost, 346 -> 387.
+constexpr int kAheadWarps = 8;
+template <typename TX, typename TV, int T, bool COHERENT = false>
+__device__ __forceinline__ void segment_partial_ahead(const int32_t* __restrict__ col, const TV* __restrict__ val,
+                                                      const TX* __restrict__ X, int64_t ldx, int s, int e, int lane,
+                                                      float* acc) {
+    constexpr int U = 16, V = Pack<TX>::V, TPW = 32 / T;
+#pragma unroll
+    for (int v = 0; v < V; ++v) acc[v] = 0.f;
+    int j = s + lane / T;
+    int32_t c[U];
+    TV w[U];
+    bool more = j + (U - 1) * TPW < e;
+    if (more) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) { c[u] = ld_stream_i32(col + j + u * TPW); w[u] = ld_stream_val<TV>(val + j + u * TPW); }
+    }
+    while (more) {
+        uint4 x[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) x[u] = ld_row<COHERENT>(X + int64_t(c[u]) * ldx);
+        j += U * TPW;
+        more = j + (U - 1) * TPW < e;
+        TV wn[U];
+        if (more) {
+#pragma unroll
+            for (int u = 0; u < U; ++u) { c[u] = ld_stream_i32(col + j + u * TPW); wn[u] = ld_stream_val<TV>(val + j + u * TPW); }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) axpy_vec<TX, TV>(w[u], x[u], acc);
+        if (more) {
+#pragma unroll
+            for (int u = 0; u < U; ++u) w[u] = wn[u];
+        }
+    }
+    if (j + 7 * TPW < e) {
+        segment_tail<8, TX, TV, TPW, COHERENT>(col, val, X, ldx, j, acc);
+        j += 8 * TPW;
+    }
+    segment_rest<TX, TV, TPW, COHERENT>(col, val, X, ldx, j, e, acc);
+}
+
+inline bool seg_ahead(int64_t n_seg, int sm_count) { return n_seg <= int64_t(sm_count) * kAheadWarps; }
 
 // One gather round of a row staged in shared memory: the R entries base..base+R-1 (column
 // and value from shared memory), their 16-byte X gathers issued together, then accumulated
