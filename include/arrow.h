@@ -182,7 +182,7 @@ void arrow_free(arrow_handle h);
  * X is permuted into the first level's order once, every step runs the split head-row
  * reduction and the fused arrow-row kernel (all levels, fixed level order, no atomics),
  * and the result is permuted back once (Section 5.1: rows stay in pi_0 order between
- * iterations).  sigma (Section 2 leaves it to the application) is composed from three
+ * iterations): by the last iteration's stores, or with ARROW_RESCALE in a pass of its own.  sigma (Section 2 leaves it to the application) is composed from three
  * optional parts in a fixed order, sigma(Y) = colnorm(rownorm(relu(Y))):
  *   ARROW_RELU    -- max(0, y) on every element (the non-linearity of a graph-network
  *                    layer, the use the introduction motivates), fused into the row store;

@@ -7,7 +7,8 @@
 //      (two pi_0-ordered feature buffers + split-row partials) fits the HBM budget,
 //   3. launches ONE iteration for every active request: the permute-in of the newly admitted,
 //      one launch per kernel class (split-row segments, rows, combine) over the work units of
-//      all active requests, and the permute-out of those that just did their last iteration.
+//      all active requests; the last iteration of a request stores into its Y (narrow rows keep a
+//      permute-out).
 // Requests that arrive while others are on the GPU join at the next step; their work shares
 // the launches.  Every request keeps its own ping-pong parity, and the per-row arithmetic is
 // that of arrow_spmm, so a request gives the same bits alone or in any mix.

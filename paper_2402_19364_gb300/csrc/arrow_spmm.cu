@@ -17,7 +17,8 @@
 //                head-row reduction, Alg. 1 line 3).  With rescaling it also emits FP64
 //                per-column sums of squares of the rows it wrote.
 //     finalize   d_t[j] = 1 / sqrt(sum of the FP64 partials of column j), fixed order.
-//   permute-out  Y[v] = X^[pi_0(v)] (* d_T with rescaling)
+//   permute-out  Y[v] = X^[pi_0(v)] (* d_T with rescaling); without rescaling the last step stores its
+//                rows there itself
 //
 // Every accumulation has a fixed order, so repeated calls are bit-identical.
 #include <cuda_bf16.h>
@@ -1058,7 +1059,10 @@ static bool fused_eligible(const arrow_handle_s* h, int64_t k, int x_dtype) {
     return h->n <= (int64_t(1) << 20) && h->nnz <= (int64_t(8) << 20);
 }
 
-static int make_plan(const arrow_handle_s* h, int64_t k, int x_dtype, int flags, Plan& p) {
+// `share`: let CTAs share a tile's rows (row_parts).  With the rescale every CTA has a slot of FP64
+// column sums, so this is what makes a small problem's workspace larger; without it the size is
+// that of one CTA per tile.
+static int make_plan(const arrow_handle_s* h, int64_t k, int x_dtype, int flags, Plan& p, bool share = true) {
     p.V = int(16 / dtype_size(x_dtype));
     if (k % p.V) { set_error("arrow_spmm: k * sizeof(dtype) must be a multiple of 16 bytes"); return ARROW_EINVAL; }
     int64_t t = k / p.V;
@@ -1080,7 +1084,7 @@ static int make_plan(const arrow_handle_s* h, int64_t k, int x_dtype, int flags,
     const int64_t n_tiles = h->tile_row.empty() ? 0 : int64_t(h->tile_row.size()) - 1;
     const int cap = (flags & ARROW_RESCALE) ? ARROW_ROWS_MIN_BLOCKS_RESCALE : ARROW_ROWS_MIN_BLOCKS;
     const int64_t most = int64_t(sm) * std::min(h->tune.ctas_per_sm, cap);
-    p.parts = row_parts(n_tiles, most, h->tune.tile_rows, 256 / p.T);
+    p.parts = share ? row_parts(n_tiles, most, h->tune.tile_rows, 256 / p.T) : 1;
     p.rows_grid = int(std::max<int64_t>(1, std::min<int64_t>(n_tiles * p.parts, most)));
     const int64_t n_long = int64_t(h->long_rows.size());
     const int64_t teams = 256 / p.T;
@@ -1570,6 +1574,8 @@ int arrow_spmm_ws(arrow_handle h, const void* X, int64_t k, int32_t iters, void*
     if (h->n == 0 || k == 0) return ARROW_OK;
     Plan p;
     if ((rc = make_plan(h, k, x_dtype, flags, p))) return rc;
+    // a workspace with room for one CTA per tile only is still enough
+    if (iters > 0 && ws_bytes < p.total && (rc = make_plan(h, k, x_dtype, flags, p, false))) return rc;
     if (iters > 0 && (!workspace || ws_bytes < p.total || (reinterpret_cast<uintptr_t>(workspace) & 255))) {
         set_error("arrow_spmm_ws: workspace missing, too small or not 256-byte aligned");
         return ARROW_EINVAL;
@@ -1610,6 +1616,7 @@ int arrow_spmm_static(arrow_handle h, const void* X, int64_t k, int32_t iters, v
     if (h->n == 0 || k == 0) return ARROW_OK;
     Plan p;
     if ((rc = make_plan(h, k, x_dtype, flags, p))) return rc;
+    if (p.total > kStaticScratchBytes && (rc = make_plan(h, k, x_dtype, flags, p, false))) return rc;
     if (iters > 0 && p.total > kStaticScratchBytes) {
         set_error("arrow_spmm_static: this problem needs " + std::to_string(p.total) +
                   " bytes of scratch, more than the library's static " + std::to_string(kStaticScratchBytes) +

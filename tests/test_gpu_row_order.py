@@ -50,3 +50,23 @@ def test_rows_by_length(arrow, tile, k):
     for got in (M.spmm(Xd, 1), arrow.ArrowBatch([M]).spmm([Xd], 1)[0]):
         Y = got.cpu().numpy().astype(np.float64)
         assert np.all(np.abs(Y - R) <= 1e-5 * np.max(R, axis=0))
+
+
+@pytest.mark.parametrize("k,rescale", [(16, True), (128, True), (16, False)])
+def test_smaller_workspace_still_taken(arrow, k, rescale):
+    """A workspace with FP64 sums for one CTA per tile only (less than workspace_size asks for where
+    several CTAs share a tile) is accepted and gives the result of the full one."""
+    A = w.grid_stencil((40, 37), seed=3)
+    M = arrow.ArrowMatrix(A, 40)
+    X = torch.from_numpy(w.features(A.n, k, seed=4)).cuda()
+    full = M.workspace_size(k, "f32", rescale)
+    rows = -(-A.n * k * 4 // 256) * 256
+    one = 2 * rows + -(-k * 4 // 256) * 256                      # features, (no) segment partials
+    if rescale:
+        one += -(-M.stats()["tiles"] * k * 8 // 256) * 256 + -(-2 * k * 8 // 256) * 256
+    assert one <= full and (one < full or not rescale)
+    Y = M.spmm(X, 3, rescale=rescale)
+    Yw = M.spmm_ws(X, 3, torch.empty(one, dtype=torch.uint8, device="cuda"), rescale=rescale)
+    assert torch.allclose(Y, Yw, rtol=0, atol=1e-5 * 3 * float(Y.abs().max()))
+    with pytest.raises(arrow.ArrowError):
+        M.spmm_ws(X, 3, torch.empty(one - 256, dtype=torch.uint8, device="cuda"), rescale=rescale)
