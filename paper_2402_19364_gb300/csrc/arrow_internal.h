@@ -127,6 +127,7 @@ struct arrow_handle_s {
     arrow_tuning tune{arrow::kTileRows, arrow::kTileNnz, 4, 70, 0, 0};
     double decompose_seconds = 0.0;
     bool uploaded = false;
+    bool long_desc = true;   // some short row has more entries than its descriptor holds (kLongDesc)
     // bumped whenever the device arrays or the tile table change (upload, re-tiling):
     // batches that cached descriptors or work-unit counts of this handle rebuild them
     uint64_t generation = 0;

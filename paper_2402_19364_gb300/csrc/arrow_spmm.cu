@@ -67,7 +67,7 @@ void set_error(const std::string& msg) { g_last_error = msg; }
 static inline int rows_smem_bytes(const TileLayout& L, int norm_doubles) { return 128 + kStages * L.buf + 8 * norm_doubles; }
 
 struct RowArgs {
-    const int32_t* rowptr;     // short-row stream
+    const int32_t* long_rowptr;   // row pointers, for rows of kLongDesc entries or more; null if there are none
     const uint32_t* row_desc;
     const int32_t* col;
     const void* val;
@@ -216,10 +216,11 @@ __global__ void __launch_bounds__(256, RESCALE ? ARROW_ROWS_MIN_BLOCKS_RESCALE :
         const int step = TEAMS * a.parts;
         uint32_t dn = sdesc[min(q0, nrows)];
         for (int q = q0; q < nrows; q += step) {
-            const RowDesc rd = row_desc_unpack(dn, a.rowptr, r0);
+            const RowDesc rd = row_desc_unpack(dn, a.long_rowptr, r0);
             dn = sdesc[min(q + step, nrows)];
             const int s = rd.start, e = rd.start + rd.len;
-            const int64_t yr0 = a.out_idx ? __ldg(a.out_idx + r0 + rd.row) : r0 + rd.row;
+            // (with the rescale the permute-out is never folded in)
+            const int64_t yr0 = !RESCALE && a.out_idx ? __ldg(a.out_idx + r0 + rd.row) : r0 + rd.row;
             float acc[V];
 #pragma unroll
             for (int v = 0; v < V; ++v) acc[v] = 0.f;
@@ -928,6 +929,9 @@ static int build_row_desc(arrow_handle_s* h) {
         d.bytes += bytes;
         ACK(cudaMemset(reinterpret_cast<char*>(d.row_desc) + size_t(h->n) * sizeof(uint32_t), 0, kPad));
     }
+    h->long_desc = false;
+    for (int64_t r = 0; r < h->n && !h->long_desc; ++r)
+        h->long_desc = h->f_rowptr[r + 1] - h->f_rowptr[r] >= int32_t(kLongDesc);
     const int grid = int(std::min<int64_t>(n_tiles, int64_t(d.sm_count) * 16));
     arrow_row_desc_kernel<<<grid, 256>>>(d.rowptr, d.tile_row, int(n_tiles), d.row_desc);
     ACK(cudaGetLastError());
@@ -1134,7 +1138,7 @@ static void launch_step(const arrow_handle_s* h, const Plan& p, const TX* cur, T
             pf.end(ARROW_K_SEGMENTS, e0);
         }
         const TileLayout L = tile_layout(h->tune.tile_rows, h->tune.tile_nnz);
-        RowArgs ra{d.rowptr, d.row_desc, col, d.val, d.tile_row, d.tile_ent, n_tiles, p.parts, cur, nxt, k, koff, p.kc, scale_in, np,
+        RowArgs ra{h->long_desc ? d.rowptr : nullptr, d.row_desc, col, d.val, d.tile_row, d.tile_ent, n_tiles, p.parts, cur, nxt, k, koff, p.kc, scale_in, np,
                    d.status, out_idx, L.rp, L.col, L.buf, sigma};
         const int smem = rows_smem_bytes(L, np ? 8 * p.kc : 0);
         cudaEvent_t e0 = pf.begin();
