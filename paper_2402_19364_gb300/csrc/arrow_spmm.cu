@@ -452,8 +452,11 @@ __global__ void __launch_bounds__(256) arrow_norm_finalize_kernel(const double* 
                                                                   double* scale_out) {
     const int64_t c = blockIdx.x;
     double t = 0.0;
+    // The next rows kernel starts at this kernel's end only: coming in while these few CTAs hold shared
+    // memory, its persistent CTAs were placed unevenly for their whole life (256^3 grid, 3 CTAs per
+    // SM at a 60 % carveout, 10 iterations: 8.82 ms per call against 7.48; default tiles 7.69
+    // against 7.59), for 1.5 us less per launch on a 100^3 grid.
     pdl_wait();
-    pdl_launch();
     for (int p = threadIdx.x; p < nparts; p += blockDim.x) t += partials[int64_t(p) * k + c];
     __shared__ double sh[256];
     sh[threadIdx.x] = t;

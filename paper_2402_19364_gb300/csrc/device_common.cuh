@@ -144,8 +144,8 @@ __device__ __forceinline__ void axpy_vec<float, float>(float w, const uint4& x, 
 // during a call, and lets the next kernel start only after that (pdl_launch(), or its end), so at
 // most two kernels overlap and a kernel's completion implies that of all before it.
 // What it takes off a launch: 64 x 64 grid, 10 iterations 67.6 -> 48.4 us per call; 100^3 grid, 20
-// iterations with the rescale 1174 -> 1046; R-MAT 16 FP32, 3 iterations 184 -> 161; 24-matrix FP16
-// batch 1974 -> 1960.  The gather, segment and combine kernels fill the SMs and let the next start
+// iterations with the rescale 1174 -> 1067; R-MAT 16 FP32, 3 iterations 184 -> 161; 24-matrix FP16
+// batch 1974 -> 1960.  The gather, segment, combine and norm kernels let the next start
 // at their end only: a rows kernel that came in while a permute was running cost 8 us (BF16 layer
 // 61.5 -> 69.5 us) and R-MAT 16 went from 161 to 178.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
