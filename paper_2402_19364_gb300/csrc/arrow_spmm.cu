@@ -1659,6 +1659,9 @@ int arrow_set_tuning(arrow_handle h, const arrow_tuning* t) {
         return ARROW_EINVAL;
     }
     const bool retile = t->tile_rows != h->tune.tile_rows || t->tile_nnz != h->tune.tile_nnz;
+    // batches pick the new tile tables and launch shape up; compared before build_tiles, which stores the
+    // new shape in h->tune, and bumped before any table is replaced
+    if (std::memcmp(&h->tune, t, sizeof(*t)) != 0) h->generation++;
     if (retile) {
         build_tiles(h, t->tile_rows, t->tile_nnz);
         if (h->uploaded) {
@@ -1677,7 +1680,6 @@ int arrow_set_tuning(arrow_handle h, const arrow_tuning* t) {
         int rc = upload_vertex_cols(h);
         if (rc) return rc;
     }
-    if (std::memcmp(&h->tune, t, sizeof(*t)) != 0) h->generation++;   // batches pick the new launch shape up
     h->tune = *t;
     return ARROW_OK;
 }

@@ -1,0 +1,247 @@
+// Host logic of the library on a fake CUDA runtime (no GPU): the library's own objects linked with
+// the runtime functions below, which keep "device" memory on the host and launch nothing, but
+// record where every allocation, copy, clear and launch went.  Two devices.  A freed block is never
+// reused, so a pointer into one is recognised.  Prints "ok" or the first check that failed.
+//
+// usage: fake_cuda_check <check>
+#include <cuda_runtime_api.h>
+
+#include <cstdint>
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+#include <map>
+#include <string>
+#include <vector>
+
+#include "arrow.h"
+
+// ---- the fake runtime ----------------------------------------------------------------------
+namespace {
+struct Block { char* p; size_t bytes; int dev; bool freed; };
+struct Launch { std::string name; int dev; cudaStream_t stream; std::vector<char> arg0; };
+struct Clear { char* p; size_t bytes; cudaStream_t stream; };
+std::vector<Block> g_blocks;
+std::vector<Launch> g_launches;
+std::vector<Clear> g_clears;
+std::map<const void*, std::string> g_names;
+thread_local int g_dev = 0;
+int g_fail_malloc = -1;        // the number of the cudaMalloc that fails from here on (0: the next)
+int g_instantiated = 0;
+constexpr size_t kArgBytes = 64;   // of a kernel's first argument that are kept (every argument struct is larger)
+
+Block* find(const void* p) {
+    for (Block& b : g_blocks)
+        if (p >= b.p && p < b.p + b.bytes) return &b;
+    return nullptr;
+}
+void record(const void* fn, void** args, cudaStream_t s) {
+    Launch l{g_names.count(fn) ? g_names[fn] : "?", g_dev, s, {}};
+    if (l.name.find("arrow_rows") != std::string::npos || l.name.find("arrow_batch") != std::string::npos ||
+        l.name.find("arrow_fused") != std::string::npos)
+        l.arg0.assign(static_cast<char*>(args[0]), static_cast<char*>(args[0]) + kArgBytes);
+    g_launches.push_back(l);
+}
+int g_token = 0;
+template <class T>
+cudaError_t token(T* out) {   // a handle that nobody dereferences
+    *out = reinterpret_cast<T>(uintptr_t(++g_token) * 16);
+    return cudaSuccess;
+}
+}  // namespace
+
+extern "C" {
+void** __cudaRegisterFatBinary(void*) { static void* h; return &h; }
+void __cudaRegisterFatBinaryEnd(void**) {}
+void __cudaUnregisterFatBinary(void**) {}
+void __cudaRegisterFunction(void**, const char* fn, char*, const char* name, int, uint3*, uint3*, dim3*, dim3*, int*) {
+    g_names[fn] = name;
+}
+void __cudaRegisterVar(void**, char*, char*, const char*, int, size_t, int, int) {}
+cudaError_t __cudaGetKernel(cudaKernel_t* k, const void* fn) {
+    *k = reinterpret_cast<cudaKernel_t>(const_cast<void*>(fn));
+    return cudaSuccess;
+}
+struct Config { dim3 g, b; size_t smem; void* s; } g_config;
+unsigned __cudaPushCallConfiguration(dim3 g, dim3 b, size_t smem, void* s) { g_config = {g, b, smem, s}; return 0; }
+cudaError_t __cudaPopCallConfiguration(dim3* g, dim3* b, size_t* smem, void* s) {
+    *g = g_config.g; *b = g_config.b; *smem = g_config.smem;
+    *static_cast<void**>(s) = g_config.s;
+    return cudaSuccess;
+}
+cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3, void** args, size_t, cudaStream_t s) {
+    record(reinterpret_cast<const void*>(k), args, s);
+    return cudaSuccess;
+}
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* fn, void** args) {
+    record(fn, args, c->stream);
+    return cudaSuccess;
+}
+cudaError_t cudaLaunchCooperativeKernel(const void* fn, dim3, dim3, void** args, size_t, cudaStream_t s) {
+    record(fn, args, s);
+    return cudaSuccess;
+}
+cudaError_t cudaGetDevice(int* d) { *d = g_dev; return cudaSuccess; }
+cudaError_t cudaSetDevice(int d) { g_dev = d; return cudaSuccess; }
+cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr a, int) {
+    *v = a == cudaDevAttrMultiProcessorCount ? 8 : 1;
+    return cudaSuccess;
+}
+cudaError_t cudaMalloc(void** p, size_t bytes) {
+    if (g_fail_malloc >= 0 && g_fail_malloc-- == 0) return cudaErrorMemoryAllocation;
+    char* q = static_cast<char*>(std::aligned_alloc(256, (bytes + 511) / 256 * 256));
+    std::memset(q, 0, bytes);
+    g_blocks.push_back({q, bytes, g_dev, false});
+    *p = q;
+    return cudaSuccess;
+}
+cudaError_t cudaFree(void* p) {
+    if (Block* b = find(p)) b->freed = true;
+    return cudaSuccess;
+}
+cudaError_t cudaHostAlloc(void** p, size_t bytes, unsigned) { *p = std::calloc(1, bytes); return cudaSuccess; }
+cudaError_t cudaFreeHost(void*) { return cudaSuccess; }
+cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) { std::memcpy(d, s, n); return cudaSuccess; }
+cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) {
+    std::memmove(d, s, n);
+    return cudaSuccess;
+}
+cudaError_t cudaMemset(void* p, int v, size_t n) { std::memset(p, v, n); return cudaSuccess; }
+cudaError_t cudaMemsetAsync(void* p, int v, size_t n, cudaStream_t s) {
+    g_clears.push_back({static_cast<char*>(p), n, s});
+    std::memset(p, v, n);
+    return cudaSuccess;
+}
+cudaError_t cudaGetSymbolAddress(void** p, const void* symbol) { *p = const_cast<void*>(symbol); return cudaSuccess; }
+cudaError_t cudaGetDriverEntryPointByVersion(const char*, void** f, unsigned, unsigned long long,
+                                             cudaDriverEntryPointQueryResult* q) {
+    *f = nullptr;
+    *q = cudaDriverEntryPointSymbolNotFound;
+    return cudaSuccess;
+}
+cudaError_t cudaDeviceSynchronize() { return cudaSuccess; }
+cudaError_t cudaGetLastError() { return cudaSuccess; }
+const char* cudaGetErrorString(cudaError_t) { return "fake error"; }
+cudaError_t cudaFuncSetAttribute(const void*, cudaFuncAttribute, int) { return cudaSuccess; }
+cudaError_t cudaEventCreate(cudaEvent_t* e) { return token(e); }
+cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) { return token(e); }
+cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaEventQuery(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) { *ms = 1.f; return cudaSuccess; }
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { return token(s); }
+cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) { return cudaSuccess; }
+cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t* g) { return token(g); }
+cudaError_t cudaGraphInstantiate(cudaGraphExec_t* e, cudaGraph_t, unsigned long long) { ++g_instantiated; return token(e); }
+cudaError_t cudaGraphDestroy(cudaGraph_t) { return cudaSuccess; }
+cudaError_t cudaGraphExecDestroy(cudaGraphExec_t) { return cudaSuccess; }
+cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t) { return cudaSuccess; }
+}
+
+// ---- the checks ----------------------------------------------------------------------------
+namespace {
+#define CHECK(cond)                                                              \
+    do {                                                                         \
+        if (!(cond)) { std::printf("line %d: %s\n", __LINE__, #cond); return 1; } \
+    } while (0)
+#define OK(call)                                                                                                    \
+    do {                                                                                                            \
+        if (int rc_ = (call)) { std::printf("line %d: %s = %d (%s)\n", __LINE__, #call, rc_, arrow_last_error()); return 1; } \
+    } while (0)
+
+// A ring of n vertices with self-loops, each vertex also joined to `hubs` hubs (rows that are split).
+arrow_handle make(int64_t n, int hubs, int device = -1) {
+    std::vector<std::map<int32_t, double>> rows(n);
+    for (int64_t v = 0; v < n; ++v)
+        for (int64_t u : {v, (v + 1) % n, (v + n - 1) % n}) rows[v][int32_t(u)] = rows[u][int32_t(v)] = 1.0 + double(v % 3);
+    for (int h = 0; h < hubs; ++h)
+        for (int64_t v = 0; v < n; ++v) rows[v][h] = rows[h][int32_t(v)] = 0.5;
+    std::vector<int64_t> rp{0};
+    std::vector<int32_t> ci;
+    std::vector<double> va;
+    for (auto& r : rows) {
+        for (auto& e : r) { ci.push_back(e.first); va.push_back(e.second); }
+        rp.push_back(int64_t(ci.size()));
+    }
+    arrow_csr A{};
+    A.n = n; A.nnz = int64_t(ci.size()); A.rowptr = rp.data(); A.colidx = ci.data(); A.values = va.data();
+    arrow_opts o;
+    arrow_opts_default(&o);
+    o.device = device;
+    o.nthreads = 1;
+    arrow_handle h = nullptr;
+    return arrow_decompose(&A, 16, &o, &h) == ARROW_OK ? h : nullptr;
+}
+
+char* buffer(size_t bytes) {
+    void* p = nullptr;
+    return cudaMalloc(&p, bytes) == cudaSuccess ? static_cast<char*>(p) : nullptr;
+}
+
+// No launch of a batch kernel since `from` has a descriptor that points into freed memory (the kernels'
+// first argument starts with the pointer to the descriptors).
+int stale_descriptors(size_t from) {
+    int bad = 0;
+    for (size_t i = from; i < g_launches.size(); ++i) {
+        if (g_launches[i].name.find("arrow_batch") == std::string::npos) continue;
+        char* d = nullptr;
+        std::memcpy(&d, g_launches[i].arg0.data(), sizeof(d));
+        const Block* b = find(d);
+        if (!b || b->freed) { ++bad; continue; }
+        for (size_t o = 0; o + 8 <= b->bytes; o += 8) {
+            void* w = nullptr;
+            std::memcpy(&w, b->p + o, 8);
+            const Block* t = find(w);
+            if (t && t->freed) ++bad;
+        }
+    }
+    return bad;
+}
+
+// A batch made before a member is re-tiled walks the new tile tables, whatever part of the tuning
+// changed, and captures its graph again.
+int retiled_member() {
+    arrow_handle h[2] = {make(700, 2), make(300, 0)};
+    CHECK(h[0] && h[1]);
+    arrow_batch B = nullptr;
+    OK(arrow_batch_create(h, 2, &B));
+    const int64_t k[2] = {8, 16};
+    const void* X[2] = {buffer(700 * 8 * 4), buffer(300 * 16 * 4)};
+    void* Y[2] = {buffer(700 * 8 * 4), buffer(300 * 16 * 4)};
+    OK(arrow_batch_spmm(B, X, Y, k, 3, ARROW_F32, 0, nullptr));
+    OK(arrow_batch_spmm(B, X, Y, k, 3, ARROW_F32, ARROW_GRAPH, nullptr));
+    const arrow_tuning shapes[] = {{512, 4096, 4, 70, 0, 0}, {512, 2048, 4, 70, 0, 0}, {64, 2048, 4, 70, 0, 0},
+                                   {64, 2048, 3, 70, 0, 0}, {64, 1024, 3, 50, 0, 0}};
+    for (const arrow_tuning& t : shapes)
+        for (arrow_handle m : h) {
+            OK(arrow_set_tuning(m, &t));
+            const size_t from = g_launches.size();
+            const int graphs = g_instantiated;
+            OK(arrow_batch_spmm(B, X, Y, k, 3, ARROW_F32, 0, nullptr));
+            OK(arrow_batch_spmm(B, X, Y, k, 3, ARROW_F32, ARROW_GRAPH, nullptr));
+            CHECK(g_launches.size() > from);
+            CHECK(stale_descriptors(from) == 0);
+            CHECK(g_instantiated == graphs + 1);
+        }
+    // the same tuning again changes nothing: the graph is replayed
+    const int graphs = g_instantiated;
+    OK(arrow_set_tuning(h[0], &shapes[4]));
+    OK(arrow_batch_spmm(B, X, Y, k, 3, ARROW_F32, ARROW_GRAPH, nullptr));
+    CHECK(g_instantiated == graphs);
+    return 0;
+}
+
+}  // namespace
+
+int main(int argc, char** argv) {
+    const std::string which = argc > 1 ? argv[1] : "";
+    const std::map<std::string, int (*)()> checks{{"retiled_member", retiled_member}};
+    const auto it = checks.find(which);
+    if (it == checks.end()) { std::printf("no check %s\n", which.c_str()); return 2; }
+    const int rc = it->second();
+    if (rc == 0) std::printf("ok\n");
+    return rc;
+}

@@ -149,3 +149,22 @@ def test_member_retuned_after_batch_creation(arrow):
             torch.cuda.synchronize()
             assert B.status() == 0
             assert all(torch.equal(y, r) for y, r in zip(Ys, ref))
+
+
+def test_member_retiled_with_nothing_else_changed(arrow):
+    # only rows and entries per tile change: the tables the batch's descriptors point to are
+    # replaced, and the order of the rows inside a tile with them
+    mats, ks = _rgg_batch(4, 22)
+    ms = [arrow.ArrowMatrix(A, int(np.ceil(np.sqrt(A.n))), value_dtype="f16") for A in mats]
+    Xs = [torch.from_numpy(w.features(A.n, k, seed=i)).to("cuda", torch.float16) for i, (A, k) in enumerate(zip(mats, ks))]
+    B = arrow.ArrowBatch(ms)
+    ref = [y.clone() for y in B.spmm(Xs, 3, graph=True)]
+    t = ms[0].tuning
+    for rows, entries in ((512, 4096), (512, 2048), (128, 1024)):
+        for M in ms:
+            M.set_tuning(rows, entries, t["ctas_per_sm"], t["carveout"])
+        for graph in (False, True):
+            Ys = B.spmm(Xs, 3, graph=graph)
+            torch.cuda.synchronize()
+            assert B.status() == 0
+            assert all(torch.equal(y, r) for y, r in zip(Ys, ref))
