@@ -205,12 +205,16 @@ void arrow_free(arrow_handle h);
 int arrow_spmm(arrow_handle h, const void* X, int64_t k, int32_t iters, void* Y,
                int32_t x_dtype, int32_t flags, void* stream);
 
-/* Workspace bytes arrow_spmm_ws needs for (k, x_dtype, flags). */
+/* Workspace bytes arrow_spmm_ws needs for (k, x_dtype, flags) under the handle's current tuning. */
 int arrow_workspace_size(arrow_handle h, int64_t k, int32_t x_dtype, int32_t flags, size_t* bytes);
 
 /* arrow_spmm with caller-provided DEVICE workspace (256-byte aligned, >= the size from
  * arrow_workspace_size).  Makes no allocation; calls with distinct workspaces on
- * distinct streams may overlap on one handle (the handle's device data is read-only). */
+ * distinct streams may overlap on one handle (its device data is read-only but for the status
+ * word).  A smaller workspace is taken too where the call can do with less (one CTA per tile, or no
+ * one-launch path): without ARROW_RESCALE the result is the same bits, with it the FP64 column
+ * sums are then grouped differently (rounding).  Errors: as arrow_spmm; ARROW_EINVAL if it is too
+ * small for any form. */
 int arrow_spmm_ws(arrow_handle h, const void* X, int64_t k, int32_t iters, void* Y,
                   int32_t x_dtype, int32_t flags, void* workspace, size_t ws_bytes, void* stream);
 
@@ -222,7 +226,7 @@ int arrow_spmm_ws(arrow_handle h, const void* X, int64_t k, int32_t iters, void*
  * and result as arrow_spmm (X, Y on the device, caller-owned), but the scratch lives in one
  * file-scope device array of 64 MiB that every GPU loading the library holds until the
  * process exits.  Problems whose scratch (two n x k feature buffers, split-row partials,
- * FP64 norm sums: the arrow_workspace_size value) exceeds 64 MiB -- about 500,000 rows at
+ * FP64 norm sums: as for arrow_spmm_ws) exceeds 64 MiB in every form -- about 500,000 rows at
  * k = 16 in FP32 -- are rejected with ARROW_EINVAL.  The call allocates nothing.  The
  * handle's device must be current.  The first call in each CUDA context looks up the
  * array's device address (cudaGetSymbolAddress) and caches it for that context: make that

@@ -995,7 +995,7 @@ static int upload_to_current(arrow_handle_s* h) {
     if ((rc = upload_vec(&d.long_segptr, h->long_segptr, d.bytes))) return rc;
     if ((rc = upload_vec(&d.seg_begin, h->seg_begin, d.bytes))) return rc;
     if ((rc = upload_vec(&d.seg_end, h->seg_end, d.bytes))) return rc;
-    if ((rc = upload_vec(&d.status, std::vector<int32_t>(4, 0), d.bytes))) return rc;
+    if ((rc = upload_vec(&d.status, std::vector<int32_t>(1, 0), d.bytes))) return rc;
     const int64_t n = h->n;
     {
         std::vector<int32_t> perm0(n), iperm0(n);
@@ -1022,6 +1022,7 @@ struct Plan {
     int rows_grid;   // CTAs of the rows kernel (= its FP64 norm partial slots)
     int comb_grid;   // CTAs of the combine kernel (= its partial slots after the rows kernel's)
     size_t x_bytes, part_bytes, np_bytes, sc_bytes, total;
+    size_t bar_off;  // the one-launch path's arrival count, from the start of the segment partials
 };
 
 // Shared-memory opt-in and carveout of a kernel, cached per (device, kernel): both are
@@ -1068,8 +1069,9 @@ static bool fused_eligible(const arrow_handle_s* h, int64_t k, int x_dtype) {
 
 // `share`: let CTAs share a tile's rows (row_parts).  With the rescale every CTA has a slot of FP64
 // column sums, so this is what makes a small problem's workspace larger; without it the size is
-// that of one CTA per tile.
-static int make_plan(const arrow_handle_s* h, int64_t k, int x_dtype, int flags, Plan& p, bool share = true) {
+// that of one CTA per tile.  `one_launch`: let the tuning's one-launch path be taken.
+static int make_plan(const arrow_handle_s* h, int64_t k, int x_dtype, int flags, Plan& p, bool share = true,
+                     bool one_launch = true) {
     p.V = int(16 / dtype_size(x_dtype));
     if (k % p.V) { set_error("arrow_spmm: k * sizeof(dtype) must be a multiple of 16 bytes"); return ARROW_EINVAL; }
     int64_t t = k / p.V;
@@ -1102,20 +1104,32 @@ static int make_plan(const arrow_handle_s* h, int64_t k, int x_dtype, int flags,
         n_long ? int(std::max<int64_t>(1, std::min<int64_t>((n_long + teams - 1) / teams, int64_t(sm) * comb_cap))) : 0;
     const size_t sx = dtype_size(x_dtype);
     p.x_bytes = align256(size_t(h->n) * size_t(k) * sx);
-    p.part_bytes = align256(std::max<size_t>(1, h->seg_begin.size()) * size_t(p.kc) * 4);
     // the one-launch path: asked for by the tuning, for one-chunk k and small problems (where
     // kernel start-up dominates), one row per team and phase where the SMs allow (each row is a
     // chain of dependent loads, so rows per team add latency), at most one CTA per SM (all
     // resident)
     p.fused_grid = 0;
-    if (h->tune.fused_small && p.chunks == 1 && fused_eligible(h, k, x_dtype)) {
+    if (one_launch && h->tune.fused_small && p.chunks == 1 && fused_eligible(h, k, x_dtype)) {
         const int64_t per_cta = int64_t(256 / p.T);
         p.fused_grid = int(std::max<int64_t>(1, std::min<int64_t>((h->n + per_cta - 1) / per_cta, sm)));
     }
+    // its arrival count follows the partials, so that calls with workspaces of their own share none
+    p.bar_off = h->seg_begin.size() * size_t(p.kc) * 4;
+    p.part_bytes = align256(std::max(size_t(p.kc) * 4, p.bar_off + (p.fused_grid ? sizeof(unsigned) : 0)));
     const size_t np_slots = std::max<size_t>(size_t(p.rows_grid + p.comb_grid), size_t(2 * p.fused_grid));
     p.np_bytes = (flags & ARROW_RESCALE) ? align256(np_slots * size_t(k) * 8) : 0;
     p.sc_bytes = (flags & ARROW_RESCALE) ? align256(2 * size_t(k) * 8) : 0;
     p.total = 2 * p.x_bytes + p.part_bytes + p.np_bytes + p.sc_bytes;
+    return ARROW_OK;
+}
+
+// The first plan that `avail` bytes of scratch hold, or the smallest one: a workspace sized under another
+// tuning may have no room for the FP64 sums of shared tiles or for the one-launch path's count.
+static int fit_plan(const arrow_handle_s* h, int64_t k, int x_dtype, int flags, size_t avail, Plan& p) {
+    for (int form = 0; form < 4; ++form) {
+        const int rc = make_plan(h, k, x_dtype, flags, p, !(form & 1), form < 2);
+        if (rc != ARROW_OK || p.total <= avail) return rc;
+    }
     return ARROW_OK;
 }
 
@@ -1223,17 +1237,17 @@ static cudaError_t launch_fused_v(const Plan& p, FusedArgs& fa, bool rescale, cu
     }
 }
 
-// The whole call as one cooperative launch (arrow_fused_small_kernel); the barrier counter
-// is cleared on the stream first.
+// The whole call as one cooperative launch (arrow_fused_small_kernel); the barrier's arrival count, in
+// the call's own workspace, is cleared on the stream first.
 template <typename TX>
 static int launch_fused(const arrow_handle_s* h, const Plan& p, const void* X, int64_t k, int iters, void* Y, int flags,
                         char* ws, float* part, double* np, cudaStream_t s, Prof& pf) {
     const DeviceData& d = h->dev;
+    unsigned* bar = reinterpret_cast<unsigned*>(reinterpret_cast<char*>(part) + p.bar_off);
     FusedArgs fa{d.rowptr, d.col, d.val, d.lcol, d.lval, d.seg_begin, d.seg_end, d.long_rows, d.long_segptr, d.perm0,
                  d.iperm0, h->n, int64_t(h->seg_begin.size()), int64_t(h->long_rows.size()), X, Y, ws,
-                 ws + p.x_bytes, part, np, k, iters, sigma_of(flags), reinterpret_cast<unsigned*>(d.status + 2),
-                 d.status};
-    ACK(cudaMemsetAsync(d.status + 2, 0, sizeof(int32_t), s));
+                 ws + p.x_bytes, part, np, k, iters, sigma_of(flags), bar, d.status};
+    ACK(cudaMemsetAsync(bar, 0, sizeof(unsigned), s));
     cudaEvent_t e0 = pf.begin();
     cudaError_t e;
     const bool rescale = flags & ARROW_RESCALE;
@@ -1580,9 +1594,7 @@ int arrow_spmm_ws(arrow_handle h, const void* X, int64_t k, int32_t iters, void*
     if (rc) return rc;
     if (h->n == 0 || k == 0) return ARROW_OK;
     Plan p;
-    if ((rc = make_plan(h, k, x_dtype, flags, p))) return rc;
-    // a workspace with room for one CTA per tile only is still enough
-    if (iters > 0 && ws_bytes < p.total && (rc = make_plan(h, k, x_dtype, flags, p, false))) return rc;
+    if ((rc = fit_plan(h, k, x_dtype, flags, ws_bytes, p))) return rc;
     if (iters > 0 && (!workspace || ws_bytes < p.total || (reinterpret_cast<uintptr_t>(workspace) & 255))) {
         set_error("arrow_spmm_ws: workspace missing, too small or not 256-byte aligned");
         return ARROW_EINVAL;
@@ -1622,8 +1634,7 @@ int arrow_spmm_static(arrow_handle h, const void* X, int64_t k, int32_t iters, v
     }
     if (h->n == 0 || k == 0) return ARROW_OK;
     Plan p;
-    if ((rc = make_plan(h, k, x_dtype, flags, p))) return rc;
-    if (p.total > kStaticScratchBytes && (rc = make_plan(h, k, x_dtype, flags, p, false))) return rc;
+    if ((rc = fit_plan(h, k, x_dtype, flags, kStaticScratchBytes, p))) return rc;
     if (iters > 0 && p.total > kStaticScratchBytes) {
         set_error("arrow_spmm_static: this problem needs " + std::to_string(p.total) +
                   " bytes of scratch, more than the library's static " + std::to_string(kStaticScratchBytes) +

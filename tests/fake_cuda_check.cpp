@@ -6,6 +6,7 @@
 // usage: fake_cuda_check <check>
 #include <cuda_runtime_api.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <cstdio>
 #include <cstdlib>
@@ -201,6 +202,58 @@ int stale_descriptors(size_t from) {
     return bad;
 }
 
+// Calls of the one-launch path on one handle with workspaces of their own may overlap on the GPU, so nothing
+// that a call writes apart from Y and the status word lies outside its workspace: the grid barrier's
+// arrival count is cleared in the workspace, behind the segment partials and before the FP64 sums.
+int own_barrier_count() {
+    for (int hubs : {0, 3}) {
+        arrow_handle h = make(900, hubs);
+        CHECK(h);
+        const arrow_tuning t{256, 2048, 4, 70, 0, 1};
+        OK(arrow_set_tuning(h, &t));
+        arrow_stats st;
+        OK(arrow_get_stats(h, &st));
+        CHECK((hubs > 0) == (st.segments > 0));
+        for (int64_t k : {4, 64, 128})
+            for (int flags : {0, ARROW_RESCALE}) {
+                size_t bytes = 0;
+                OK(arrow_workspace_size(h, k, ARROW_F32, flags, &bytes));
+                const char *X = buffer(900 * k * 4), *last = nullptr;
+                char* Y = buffer(900 * k * 4);
+                for (int call = 0; call < 2; ++call) {
+                    char* ws = buffer(bytes);
+                    cudaStream_t s = reinterpret_cast<cudaStream_t>(uintptr_t(0x1000 + call));
+                    g_clears.clear();
+                    g_launches.clear();
+                    OK(arrow_spmm_ws(h, X, k, 5, Y, ARROW_F32, flags, ws, bytes, s));
+                    CHECK(g_launches.size() == 1 && g_launches[0].name.find("arrow_fused") != std::string::npos);
+                    CHECK(g_launches[0].stream == s);
+                    CHECK(g_clears.size() == 1 && g_clears[0].stream == s && g_clears[0].bytes == 4);
+                    const char* c = g_clears[0].p;
+                    CHECK(c != last);
+                    last = c;
+                    const size_t rows = size_t(900 * k * 4 + 255) / 256 * 256;
+                    CHECK(c >= ws + 2 * rows + size_t(st.segments * k * 4) && c + 4 <= ws + bytes);
+                    CHECK(uintptr_t(c) % 4 == 0);
+                    // the FP64 sums of the rescale start at the next 256-byte boundary at the earliest
+                    const size_t part = std::max(size_t(k * 4), size_t(st.segments * k * 4) + 4);
+                    CHECK(c + 4 <= ws + 2 * rows + (part + 255) / 256 * 256);
+                }
+                // a workspace without room for the count still runs the call, kernel by kernel
+                const size_t plain = 2 * (size_t(900 * k * 4 + 255) / 256 * 256) +
+                                     (size_t(std::max<int64_t>(1, st.segments) * k * 4) + 255) / 256 * 256;
+                if (!flags && plain < bytes) {
+                    g_launches.clear();
+                    OK(arrow_spmm_ws(h, X, k, 5, Y, ARROW_F32, flags, buffer(plain), plain, nullptr));
+                    CHECK(g_launches.size() > 5);
+                }
+                CHECK(flags || arrow_spmm_ws(h, X, k, 5, Y, ARROW_F32, flags, buffer(plain), plain - 256, nullptr) == ARROW_EINVAL);
+            }
+        arrow_free(h);
+    }
+    return 0;
+}
+
 // A batch made before a member is re-tiled walks the new tile tables, whatever part of the tuning
 // changed, and captures its graph again.
 int retiled_member() {
@@ -238,7 +291,7 @@ int retiled_member() {
 
 int main(int argc, char** argv) {
     const std::string which = argc > 1 ? argv[1] : "";
-    const std::map<std::string, int (*)()> checks{{"retiled_member", retiled_member}};
+    const std::map<std::string, int (*)()> checks{{"retiled_member", retiled_member}, {"own_barrier_count", own_barrier_count}};
     const auto it = checks.find(which);
     if (it == checks.end()) { std::printf("no check %s\n", which.c_str()); return 2; }
     const int rc = it->second();

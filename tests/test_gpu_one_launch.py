@@ -44,3 +44,26 @@ def test_rescale_at_every_width(arrow, dt, k, dims):
         assert np.max(np.max(np.abs(Y - R), axis=0) / np.max(np.abs(R), axis=0)) <= 1e-5 * it
     else:
         assert np.max(np.linalg.norm(Y - R, axis=0) / np.linalg.norm(R, axis=0)) <= 2e-2
+
+
+@pytest.mark.parametrize("rescale", [False, True])
+def test_overlapping_calls_on_one_handle(arrow, rescale):
+    """Calls with workspaces of their own on two streams may overlap on one handle: each counts its
+    grid barrier's arrivals in its own workspace, so every one gives the bits of a call alone."""
+    A = w.rmat_gcn(9, 16, seed=4)
+    M = arrow.ArrowMatrix(A, 32)
+    t = M.tuning
+    M.set_tuning(t["tile_rows"], t["tile_nnz"], t["ctas_per_sm"], t["carveout"], 0, 1)
+    assert M.stats()["segments"] > 0
+    X = torch.from_numpy(w.features(A.n, 32, seed=6)).cuda()
+    ref = M.spmm(X, 6, rescale=rescale)
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    ws = [torch.empty(M.workspace_size(32, "f32", rescale), dtype=torch.uint8, device="cuda") for _ in streams]
+    outs = [[torch.empty_like(X) for _ in range(20)] for _ in streams]
+    torch.cuda.synchronize()
+    for i in range(20):
+        for s, b, ys in zip(streams, ws, outs):
+            M.spmm_ws(X, 6, b, rescale=rescale, out=ys[i], stream=s)
+    torch.cuda.synchronize()
+    assert M.status() == 0
+    assert all(torch.equal(y, ref) for ys in outs for y in ys)

@@ -29,6 +29,6 @@ def check(tmp_path_factory):
     return run
 
 
-@pytest.mark.parametrize("name", ["retiled_member"])
+@pytest.mark.parametrize("name", ["retiled_member", "own_barrier_count"])
 def test_host_logic(check, name):
     check(name)
