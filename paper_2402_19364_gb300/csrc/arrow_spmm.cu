@@ -967,16 +967,17 @@ static int upload_vertex_cols(arrow_handle_s* h) {
     return ARROW_OK;
 }
 
-// Upload to opts.device (or the current device); the caller's current device is restored on
-// every return path.
-static int upload_impl(arrow_handle_s* h) {
+// fn() with device dev current (-1: whichever is); the caller's current device is restored on every
+// return path.
+template <class F>
+static int on_device(int dev, const char* what, F fn) {
     int prev = -1;
     ACK(cudaGetDevice(&prev));
-    if (h->opts.device >= 0 && h->opts.device != prev) ACK(cudaSetDevice(h->opts.device));
-    const int rc = upload_to_current(h);
-    if (h->opts.device >= 0 && h->opts.device != prev) {
+    if (dev >= 0 && dev != prev) ACK(cudaSetDevice(dev));
+    const int rc = fn();
+    if (dev >= 0 && dev != prev) {
         cudaError_t e = cudaSetDevice(prev);
-        if (rc == ARROW_OK && e != cudaSuccess) return cuda_fail(e, "arrow_upload: restoring the caller's device");
+        if (rc == ARROW_OK && e != cudaSuccess) return cuda_fail(e, what);
     }
     return rc;
 }
@@ -1427,6 +1428,34 @@ static int static_scratch_ptr(void** out) {
     return ARROW_OK;
 }
 
+// The checked tuning t on the handle, whose device (if it is uploaded) is current.
+static int apply_tuning(arrow_handle_s* h, const arrow_tuning* t) {
+    const bool retile = t->tile_rows != h->tune.tile_rows || t->tile_nnz != h->tune.tile_nnz;
+    // batches pick the new tile tables and launch shape up; compared before build_tiles, which stores the
+    // new shape in h->tune, and bumped before any table is replaced
+    if (std::memcmp(&h->tune, t, sizeof(*t)) != 0) h->generation++;
+    if (retile) {
+        build_tiles(h, t->tile_rows, t->tile_nnz);
+        if (h->uploaded) {
+            ACK(cudaDeviceSynchronize());
+            if (h->dev.tile_row) cudaFree(h->dev.tile_row);
+            if (h->dev.tile_ent) cudaFree(h->dev.tile_ent);
+            h->dev.tile_row = h->dev.tile_ent = nullptr;
+            size_t bytes = 0;
+            int rc;
+            if ((rc = upload_vec(&h->dev.tile_row, h->tile_row, bytes))) return rc;
+            if ((rc = upload_vec(&h->dev.tile_ent, h->tile_ent, bytes))) return rc;
+            if ((rc = build_row_desc(h))) return rc;
+        }
+    }
+    if (t->fold_permute_in && h->uploaded) {
+        int rc = upload_vertex_cols(h);
+        if (rc) return rc;
+    }
+    h->tune = *t;
+    return ARROW_OK;
+}
+
 }  // namespace arrow
 
 // ======================================================================================
@@ -1491,7 +1520,7 @@ int arrow_upload(arrow_handle h) {
     if (h->uploaded) return ARROW_OK;
     int rc;
     try {
-        rc = upload_impl(h);
+        rc = on_device(h->opts.device, "arrow_upload: restoring the caller's device", [&] { return upload_to_current(h); });
     } catch (const std::bad_alloc&) {
         set_error("arrow_upload: host allocation failed");
         rc = ARROW_ENOMEM;
@@ -1669,30 +1698,8 @@ int arrow_set_tuning(arrow_handle h, const arrow_tuning* t) {
         set_error("arrow_set_tuning: tile too large for shared memory");
         return ARROW_EINVAL;
     }
-    const bool retile = t->tile_rows != h->tune.tile_rows || t->tile_nnz != h->tune.tile_nnz;
-    // batches pick the new tile tables and launch shape up; compared before build_tiles, which stores the
-    // new shape in h->tune, and bumped before any table is replaced
-    if (std::memcmp(&h->tune, t, sizeof(*t)) != 0) h->generation++;
-    if (retile) {
-        build_tiles(h, t->tile_rows, t->tile_nnz);
-        if (h->uploaded) {
-            ACK(cudaDeviceSynchronize());
-            if (h->dev.tile_row) cudaFree(h->dev.tile_row);
-            if (h->dev.tile_ent) cudaFree(h->dev.tile_ent);
-            h->dev.tile_row = h->dev.tile_ent = nullptr;
-            size_t bytes = 0;
-            int rc;
-            if ((rc = upload_vec(&h->dev.tile_row, h->tile_row, bytes))) return rc;
-            if ((rc = upload_vec(&h->dev.tile_ent, h->tile_ent, bytes))) return rc;
-            if ((rc = build_row_desc(h))) return rc;
-        }
-    }
-    if (t->fold_permute_in && h->uploaded) {
-        int rc = upload_vertex_cols(h);
-        if (rc) return rc;
-    }
-    h->tune = *t;
-    return ARROW_OK;
+    if (!h->uploaded) return apply_tuning(h, t);
+    return on_device(h->dev.device, "arrow_set_tuning: restoring the caller's device", [&] { return apply_tuning(h, t); });
 }
 
 int arrow_autotune(arrow_handle h, const void* X, void* Y, int64_t k, int32_t iters, int32_t x_dtype, int32_t flags,

@@ -254,6 +254,28 @@ int own_barrier_count() {
     return 0;
 }
 
+// A handle on a device that is not current is re-tuned on its own device, and the caller's device stays.
+int tuned_on_its_device() {
+    arrow_handle h = make(700, 2, 1);
+    CHECK(h && g_dev == 0);
+    const arrow_tuning shapes[] = {{512, 4096, 4, 70, 0, 0}, {512, 4096, 3, 70, 0, 0}, {64, 1024, 3, 50, 1, 0}};
+    for (const arrow_tuning& t : shapes) {
+        const size_t blocks = g_blocks.size();
+        g_launches.clear();
+        OK(arrow_set_tuning(h, &t));
+        CHECK(g_dev == 0);
+        for (size_t i = blocks; i < g_blocks.size(); ++i) CHECK(g_blocks[i].dev == 1);
+        for (const Launch& l : g_launches) CHECK(l.dev == 1);
+        arrow_tuning got;
+        OK(arrow_get_tuning(h, &got));
+        CHECK(std::memcmp(&got, &t, sizeof(t)) == 0);
+    }
+    // out of range is still refused, with the caller's device current
+    const arrow_tuning bad{16, 4096, 3, 70, 0, 0};
+    CHECK(arrow_set_tuning(h, &bad) == ARROW_EINVAL && g_dev == 0);
+    return 0;
+}
+
 // A batch made before a member is re-tiled walks the new tile tables, whatever part of the tuning
 // changed, and captures its graph again.
 int retiled_member() {
@@ -291,7 +313,8 @@ int retiled_member() {
 
 int main(int argc, char** argv) {
     const std::string which = argc > 1 ? argv[1] : "";
-    const std::map<std::string, int (*)()> checks{{"retiled_member", retiled_member}, {"own_barrier_count", own_barrier_count}};
+    const std::map<std::string, int (*)()> checks{
+        {"retiled_member", retiled_member}, {"own_barrier_count", own_barrier_count}, {"tuned_on_its_device", tuned_on_its_device}};
     const auto it = checks.find(which);
     if (it == checks.end()) { std::printf("no check %s\n", which.c_str()); return 2; }
     const int rc = it->second();
