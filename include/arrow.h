@@ -118,7 +118,7 @@ int arrow_get_tuning(arrow_handle h, arrow_tuning* t);
 
 /* Re-tile the handle (host, O(n)) and, if uploaded, replace its device tile tables; waits for
  * the device first.  Runs on the handle's device, whichever is current, and leaves the caller's current
- * device as it was.  Errors: ARROW_EINVAL (out of range: 32 <= tile_rows <= 2048,
+ * device as it was.  On an error the handle keeps the tuning it had.  Errors: ARROW_EINVAL (out of range: 32 <= tile_rows <= 2048,
  * 1024 <= tile_nnz <= 16384, 1 <= ctas_per_sm <= 4, 0 <= carveout <= 100,
  * fold_permute_in and fused_small 0 or 1), ARROW_ENOMEM, ARROW_ECUDA. */
 int arrow_set_tuning(arrow_handle h, const arrow_tuning* t);

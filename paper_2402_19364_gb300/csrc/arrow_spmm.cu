@@ -920,9 +920,9 @@ static int upload_values(const arrow_handle_s* h, const std::vector<int32_t>& sr
 
 static int upload_to_current(arrow_handle_s* h);
 
-// Row descriptors of the handle's tiles, built on the device from the uploaded row pointers and tile
-// table (allocated once: their number does not depend on the tiling).
-static int build_row_desc(arrow_handle_s* h) {
+// Row descriptors of the handle's tiles, built on the device from the uploaded row pointers and the tile
+// table tile_row there (allocated once: their number does not depend on the tiling).
+static int build_row_desc(arrow_handle_s* h, const int32_t* tile_row) {
     DeviceData& d = h->dev;
     const int64_t n_tiles = h->tile_row.empty() ? 0 : int64_t(h->tile_row.size()) - 1;
     if (h->n == 0 || n_tiles == 0) return ARROW_OK;
@@ -936,7 +936,7 @@ static int build_row_desc(arrow_handle_s* h) {
     for (int64_t r = 0; r < h->n && !h->long_desc; ++r)
         h->long_desc = h->f_rowptr[r + 1] - h->f_rowptr[r] >= int32_t(kLongDesc);
     const int grid = int(std::min<int64_t>(n_tiles, int64_t(d.sm_count) * 16));
-    arrow_row_desc_kernel<<<grid, 256>>>(d.rowptr, d.tile_row, int(n_tiles), d.row_desc);
+    arrow_row_desc_kernel<<<grid, 256>>>(d.rowptr, tile_row, int(n_tiles), d.row_desc);
     ACK(cudaGetLastError());
     ACK(cudaDeviceSynchronize());
     return ARROW_OK;
@@ -967,17 +967,28 @@ static int upload_vertex_cols(arrow_handle_s* h) {
     return ARROW_OK;
 }
 
-// fn() with device dev current (-1: whichever is); the caller's current device is restored on every
+// fn(), with a failed host allocation in it as an error code (no exception leaves a C entry point).
+template <class F>
+static int no_throw(const char* what, F fn) {
+    try {
+        return fn();
+    } catch (const std::bad_alloc&) {
+        set_error(std::string(what) + ": host allocation failed");
+        return ARROW_ENOMEM;
+    }
+}
+
+// no_throw with device dev current (-1: whichever is); the caller's current device is restored on every
 // return path.
 template <class F>
 static int on_device(int dev, const char* what, F fn) {
     int prev = -1;
     ACK(cudaGetDevice(&prev));
     if (dev >= 0 && dev != prev) ACK(cudaSetDevice(dev));
-    const int rc = fn();
+    const int rc = no_throw(what, fn);
     if (dev >= 0 && dev != prev) {
         cudaError_t e = cudaSetDevice(prev);
-        if (rc == ARROW_OK && e != cudaSuccess) return cuda_fail(e, what);
+        if (rc == ARROW_OK && e != cudaSuccess) return cuda_fail(e, (std::string(what) + ": restoring the caller's device").c_str());
     }
     return rc;
 }
@@ -1012,7 +1023,7 @@ static int upload_to_current(arrow_handle_s* h) {
     if ((rc = upload_values(h, h->f_src, &d.val, d.bytes))) return rc;
     if ((rc = upload_values(h, h->l_src, &d.lval, d.bytes))) return rc;
     if (h->tune.fold_permute_in && (rc = upload_vertex_cols(h))) return rc;
-    return build_row_desc(h);
+    return build_row_desc(h, d.tile_row);
 }
 
 // ---- launch plumbing -----------------------------------------------------------------
@@ -1428,30 +1439,51 @@ static int static_scratch_ptr(void** out) {
     return ARROW_OK;
 }
 
-// The checked tuning t on the handle, whose device (if it is uploaded) is current.
+// New tiles for the handle, whose device (if it is uploaded) is current.  The tables are built beside the
+// current ones, which stay in use when a step fails.
+static int retile(arrow_handle_s* h, int tile_rows, int tile_nnz) {
+    DeviceData& d = h->dev;
+    const arrow_tuning tune = h->tune;
+    std::vector<int32_t> row, ent;
+    row.swap(h->tile_row);
+    ent.swap(h->tile_ent);
+    int32_t *d_row = nullptr, *d_ent = nullptr;
+    size_t bytes = 0;
+    int rc = no_throw("arrow_set_tuning", [&]() -> int {
+        build_tiles(h, tile_rows, tile_nnz);
+        if (!h->uploaded) return ARROW_OK;
+        int rc1;
+        if ((rc1 = upload_vec(&d_row, h->tile_row, bytes))) return rc1;
+        if ((rc1 = upload_vec(&d_ent, h->tile_ent, bytes))) return rc1;
+        ACK(cudaDeviceSynchronize());   // nothing reads the old tables and descriptors any more
+        return build_row_desc(h, d_row);
+    });
+    if (rc) {
+        cudaFree(d_row);
+        cudaFree(d_ent);
+        row.swap(h->tile_row);
+        ent.swap(h->tile_ent);
+        h->tune = tune;
+        return rc;
+    }
+    if (h->uploaded) {
+        cudaFree(d.tile_row);
+        cudaFree(d.tile_ent);
+        d.tile_row = d_row;
+        d.tile_ent = d_ent;
+    }
+    return ARROW_OK;
+}
+
+// The checked tuning t on the handle, whose device (if it is uploaded) is current.  On an error the
+// handle keeps the tuning it had.
 static int apply_tuning(arrow_handle_s* h, const arrow_tuning* t) {
-    const bool retile = t->tile_rows != h->tune.tile_rows || t->tile_nnz != h->tune.tile_nnz;
-    // batches pick the new tile tables and launch shape up; compared before build_tiles, which stores the
-    // new shape in h->tune, and bumped before any table is replaced
+    // batches pick the new tile tables and launch shape up; bumped before any table is replaced
     if (std::memcmp(&h->tune, t, sizeof(*t)) != 0) h->generation++;
-    if (retile) {
-        build_tiles(h, t->tile_rows, t->tile_nnz);
-        if (h->uploaded) {
-            ACK(cudaDeviceSynchronize());
-            if (h->dev.tile_row) cudaFree(h->dev.tile_row);
-            if (h->dev.tile_ent) cudaFree(h->dev.tile_ent);
-            h->dev.tile_row = h->dev.tile_ent = nullptr;
-            size_t bytes = 0;
-            int rc;
-            if ((rc = upload_vec(&h->dev.tile_row, h->tile_row, bytes))) return rc;
-            if ((rc = upload_vec(&h->dev.tile_ent, h->tile_ent, bytes))) return rc;
-            if ((rc = build_row_desc(h))) return rc;
-        }
-    }
-    if (t->fold_permute_in && h->uploaded) {
-        int rc = upload_vertex_cols(h);
-        if (rc) return rc;
-    }
+    int rc;
+    if (t->fold_permute_in && h->uploaded && (rc = upload_vertex_cols(h))) return rc;
+    if ((t->tile_rows != h->tune.tile_rows || t->tile_nnz != h->tune.tile_nnz) && (rc = retile(h, t->tile_rows, t->tile_nnz)))
+        return rc;
     h->tune = *t;
     return ARROW_OK;
 }
@@ -1518,13 +1550,7 @@ int arrow_decompose(const arrow_csr* A, int64_t b, const arrow_opts* o, arrow_ha
 int arrow_upload(arrow_handle h) {
     if (!h) { set_error("arrow_upload: NULL handle"); return ARROW_EINVAL; }
     if (h->uploaded) return ARROW_OK;
-    int rc;
-    try {
-        rc = on_device(h->opts.device, "arrow_upload: restoring the caller's device", [&] { return upload_to_current(h); });
-    } catch (const std::bad_alloc&) {
-        set_error("arrow_upload: host allocation failed");
-        rc = ARROW_ENOMEM;
-    }
+    const int rc = on_device(h->opts.device, "arrow_upload", [&] { return upload_to_current(h); });
     if (rc != ARROW_OK) { free_device(h->dev); return rc; }
     h->uploaded = true;
     h->generation++;
@@ -1698,8 +1724,8 @@ int arrow_set_tuning(arrow_handle h, const arrow_tuning* t) {
         set_error("arrow_set_tuning: tile too large for shared memory");
         return ARROW_EINVAL;
     }
-    if (!h->uploaded) return apply_tuning(h, t);
-    return on_device(h->dev.device, "arrow_set_tuning: restoring the caller's device", [&] { return apply_tuning(h, t); });
+    auto apply = [&] { return apply_tuning(h, t); };
+    return h->uploaded ? on_device(h->dev.device, "arrow_set_tuning", apply) : no_throw("arrow_set_tuning", apply);
 }
 
 int arrow_autotune(arrow_handle h, const void* X, void* Y, int64_t k, int32_t iters, int32_t x_dtype, int32_t flags,

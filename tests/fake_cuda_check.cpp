@@ -39,7 +39,7 @@ Block* find(const void* p) {
 void record(const void* fn, void** args, cudaStream_t s) {
     Launch l{g_names.count(fn) ? g_names[fn] : "?", g_dev, s, {}};
     if (l.name.find("arrow_rows") != std::string::npos || l.name.find("arrow_batch") != std::string::npos ||
-        l.name.find("arrow_fused") != std::string::npos)
+        l.name.find("arrow_fused") != std::string::npos || l.name.find("arrow_segments") != std::string::npos)
         l.arg0.assign(static_cast<char*>(args[0]), static_cast<char*>(args[0]) + kArgBytes);
     g_launches.push_back(l);
 }
@@ -182,6 +182,16 @@ char* buffer(size_t bytes) {
     return cudaMalloc(&p, bytes) == cudaSuccess ? static_cast<char*>(p) : nullptr;
 }
 
+// The start of the rows kernel's argument.
+struct RowArgsHead {
+    const void *long_rowptr, *row_desc, *col, *val, *tile_row, *tile_ent;
+    int32_t n_tiles;
+};
+bool live(const void* p) {
+    Block* b = find(p);
+    return b && !b->freed;
+}
+
 // No launch of a batch kernel since `from` has a descriptor that points into freed memory (the kernels'
 // first argument starts with the pointer to the descriptors).
 int stale_descriptors(size_t from) {
@@ -276,6 +286,58 @@ int tuned_on_its_device() {
     return 0;
 }
 
+// A re-tuning that runs out of device memory leaves the handle as it was: its tuning, and tile tables
+// that the next call can read.
+int failed_retuning() {
+    for (int fold : {0})
+        for (int fail = 0; fail < 6; ++fail) {
+            arrow_handle h = make(700, 2);
+            CHECK(h);
+            arrow_tuning before, after;
+            arrow_stats st, st2;
+            OK(arrow_get_tuning(h, &before));
+            OK(arrow_get_stats(h, &st));
+            const arrow_tuning t{64, 1024, 3, 50, fold, 0};
+            g_fail_malloc = fail;
+            const int rc = arrow_set_tuning(h, &t);
+            const bool failed = g_fail_malloc < 0;
+            g_fail_malloc = -1;
+            CHECK(rc == (failed ? ARROW_ENOMEM : ARROW_OK));
+            OK(arrow_get_tuning(h, &after));
+            CHECK(std::memcmp(&after, failed ? &before : &t, sizeof(after)) == 0);
+            OK(arrow_get_stats(h, &st2));
+            CHECK((st2.tiles == st.tiles) == failed);
+            const char* X = buffer(700 * 16 * 4);
+            char* Y = buffer(700 * 16 * 4);
+            for (int again = 0; again < 2; ++again) {   // then with the tuning applied after all
+                g_launches.clear();
+                OK(arrow_spmm(h, X, 16, 2, Y, ARROW_F32, 0, nullptr));
+                int rows = 0;
+                for (const Launch& l : g_launches) {
+                    if (l.name.find("arrow_rows") == std::string::npos) continue;
+                    RowArgsHead a;
+                    std::memcpy(&a, l.arg0.data(), sizeof(a));
+                    CHECK(live(a.row_desc) && live(a.col) && live(a.val) && live(a.tile_row) && live(a.tile_ent));
+                    const size_t table = size_t(a.n_tiles + 1) * 4;
+                    CHECK(find(a.tile_row)->bytes >= table && find(a.tile_ent)->bytes >= table);
+                    ++rows;
+                }
+                CHECK(rows == 2);
+                for (const Launch& l : g_launches)
+                    if (l.name.find("arrow_segments") != std::string::npos) {
+                        const void* lcol = nullptr;   // SegArgs: seg_begin, seg_end, n_seg, lcol
+                        std::memcpy(&lcol, l.arg0.data() + 24, sizeof(lcol));
+                        CHECK(live(lcol));
+                    }
+                OK(arrow_set_tuning(h, &t));
+                OK(arrow_get_stats(h, &st2));
+                CHECK(st2.tiles != st.tiles);
+            }
+            arrow_free(h);
+        }
+    return 0;
+}
+
 // A batch made before a member is re-tiled walks the new tile tables, whatever part of the tuning
 // changed, and captures its graph again.
 int retiled_member() {
@@ -314,7 +376,8 @@ int retiled_member() {
 int main(int argc, char** argv) {
     const std::string which = argc > 1 ? argv[1] : "";
     const std::map<std::string, int (*)()> checks{
-        {"retiled_member", retiled_member}, {"own_barrier_count", own_barrier_count}, {"tuned_on_its_device", tuned_on_its_device}};
+        {"retiled_member", retiled_member}, {"own_barrier_count", own_barrier_count}, {"tuned_on_its_device", tuned_on_its_device},
+        {"failed_retuning", failed_retuning}};
     const auto it = checks.find(which);
     if (it == checks.end()) { std::printf("no check %s\n", which.c_str()); return 2; }
     const int rc = it->second();

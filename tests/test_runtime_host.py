@@ -29,6 +29,6 @@ def check(tmp_path_factory):
     return run
 
 
-@pytest.mark.parametrize("name", ["retiled_member", "own_barrier_count", "tuned_on_its_device"])
+@pytest.mark.parametrize("name", ["retiled_member", "own_barrier_count", "tuned_on_its_device", "failed_retuning"])
 def test_host_logic(check, name):
     check(name)
