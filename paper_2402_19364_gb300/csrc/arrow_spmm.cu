@@ -958,12 +958,22 @@ static int upload_vertex_cols(arrow_handle_s* h) {
         out.resize(col.size());
         for (size_t j = 0; j < col.size(); ++j) out[j] = iperm0[col[j]];
     };
-    std::vector<int32_t> tmp;
-    int rc;
-    convert(h->f_col, tmp);
-    if ((rc = upload_vec(&d.col_v, tmp, d.bytes))) return rc;
-    convert(h->l_col, tmp);
-    if ((rc = upload_vec(&d.lcol_v, tmp, d.bytes))) return rc;
+    std::vector<int32_t> col, lcol;
+    convert(h->f_col, col);
+    convert(h->l_col, lcol);
+    // both or neither: a handle with either takes the folded path
+    int32_t *col_v = nullptr, *lcol_v = nullptr;
+    size_t bytes = 0;
+    int rc = upload_vec(&col_v, col, bytes);
+    if (rc == ARROW_OK) rc = upload_vec(&lcol_v, lcol, bytes);
+    if (rc != ARROW_OK) {
+        cudaFree(col_v);
+        cudaFree(lcol_v);
+        return rc;
+    }
+    d.col_v = col_v;
+    d.lcol_v = lcol_v;
+    d.bytes += bytes;
     return ARROW_OK;
 }
 

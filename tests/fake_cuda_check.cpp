@@ -287,9 +287,9 @@ int tuned_on_its_device() {
 }
 
 // A re-tuning that runs out of device memory leaves the handle as it was: its tuning, and tile tables
-// that the next call can read.
+// and vertex-id columns that the next call can read.
 int failed_retuning() {
-    for (int fold : {0})
+    for (int fold : {0, 1})
         for (int fail = 0; fail < 6; ++fail) {
             arrow_handle h = make(700, 2);
             CHECK(h);
