@@ -932,9 +932,6 @@ static int build_row_desc(arrow_handle_s* h, const int32_t* tile_row) {
         d.bytes += bytes;
         ACK(cudaMemset(reinterpret_cast<char*>(d.row_desc) + size_t(h->n) * sizeof(uint32_t), 0, kPad));
     }
-    h->long_desc = false;
-    for (int64_t r = 0; r < h->n && !h->long_desc; ++r)
-        h->long_desc = h->f_rowptr[r + 1] - h->f_rowptr[r] >= int32_t(kLongDesc);
     const int grid = int(std::min<int64_t>(n_tiles, int64_t(d.sm_count) * 16));
     arrow_row_desc_kernel<<<grid, 256>>>(d.rowptr, tile_row, int(n_tiles), d.row_desc);
     ACK(cudaGetLastError());
@@ -1033,6 +1030,9 @@ static int upload_to_current(arrow_handle_s* h) {
     if ((rc = upload_values(h, h->f_src, &d.val, d.bytes))) return rc;
     if ((rc = upload_values(h, h->l_src, &d.lval, d.bytes))) return rc;
     if (h->tune.fold_permute_in && (rc = upload_vertex_cols(h))) return rc;
+    h->long_desc = false;
+    for (int64_t r = 0; r < h->n && !h->long_desc; ++r)
+        h->long_desc = h->f_rowptr[r + 1] - h->f_rowptr[r] >= int32_t(kLongDesc);
     return build_row_desc(h, d.tile_row);
 }
 
