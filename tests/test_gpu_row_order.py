@@ -70,3 +70,61 @@ def test_smaller_workspace_still_taken(arrow, k, rescale):
     assert torch.allclose(Y, Yw, rtol=0, atol=1e-5 * 3 * float(Y.abs().max()))
     with pytest.raises(arrow.ArrowError):
         M.spmm_ws(X, 3, torch.empty(one - 256, dtype=torch.uint8, device="cuda"), rescale=rescale)
+
+
+def _matrix_of(counts, seed):
+    rng = np.random.default_rng(seed)
+    n = counts.size
+    rowptr = np.zeros(n + 1, dtype=np.int64)
+    np.cumsum(counts, out=rowptr[1:])
+    colidx = np.concatenate([np.sort(rng.choice(n, c, replace=False)) for c in counts]).astype(np.int32)
+    vals = rng.uniform(0.5, 1.5, colidx.size).astype(np.float32).astype(np.float64)
+    return w.Csr(n, rowptr, colidx, vals)
+
+
+@pytest.mark.parametrize("case", ["rows", "entries"])
+@pytest.mark.parametrize("k", [4, 16, 128])
+def test_descriptor_fields_at_their_ends(arrow, case, k):
+    """A tile of 2048 rows (the largest row number, 2047) before one of a single row, and tiles of
+    more than 8192 entries (starts that need all their bits; 12288 entries of 512 rows at most is as
+    large as shared memory takes).  At most 100 entries a row: 100 * 2^-24 = 6e-6 of the sum."""
+    rng = np.random.default_rng(12)
+    if case == "rows":
+        A, tile = _matrix_of(rng.integers(1, 4, 2049), 13), (2048, 8192)
+    else:
+        A, tile = _matrix_of(rng.integers(0, 101, 700), 14), (512, 12288)
+    M = arrow.ArrowMatrix(A, 64, long_row=256)
+    M.set_tuning(tile[0], tile[1], 1, 100)
+    pg = M.program()
+    rows, entries = np.diff(pg["tile_row"]), np.diff(pg["tile_ent"])
+    if case == "rows":
+        assert list(rows) == [2048, 1] and np.diff(pg["rowptr"])[2047] > 0
+    else:
+        assert entries.max() > 8192 + 200
+    X = np.abs(w.features(A.n, k, seed=3))
+    Xd = torch.from_numpy(X).cuda()
+    R = S.iterate(A, X.astype(np.float64), 1)
+    for got in (M.spmm(Xd, 1), arrow.ArrowBatch([M]).spmm([Xd], 1)[0]):
+        Y = got.cpu().numpy().astype(np.float64)
+        assert np.all(np.abs(Y - R) <= 1e-5 * np.max(R, axis=0))
+
+
+@pytest.mark.parametrize("fold_in", [0, 1])
+@pytest.mark.parametrize("shift", [1, 250, -1, -250])
+def test_x_and_y_overlap_in_part(arrow, fold_in, shift):
+    """Y begins some rows into X, or X some rows into Y: every call has read its X (or keeps the
+    permute-out pass) before it stores into Y, so the result is that of buffers apart."""
+    A = w.rmat_gcn(9, 16, seed=6)
+    M = arrow.ArrowMatrix(A, 32, long_row=16, segment=64)
+    t = M.tuning
+    M.set_tuning(t["tile_rows"], t["tile_nnz"], t["ctas_per_sm"], t["carveout"], fold_in)
+    X0 = torch.from_numpy(w.features(A.n, 16, seed=7)).cuda()
+    for iters in (1, 3):
+        ref = M.spmm(X0, iters)
+        buf = torch.zeros(A.n + abs(shift), 16, device="cuda")
+        at = max(0, -shift)
+        X, Y = buf[at:at + A.n], buf[at + shift:at + shift + A.n]
+        X.copy_(X0)
+        M.spmm(X, iters, out=Y)
+        torch.cuda.synchronize()
+        assert torch.equal(Y, ref)

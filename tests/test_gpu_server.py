@@ -114,3 +114,25 @@ def test_server_argument_errors(arrow, pool):
     with pytest.raises(arrow.ArrowError):
         srv.submit(Mf, X3, X3.clone(), 1)                               # mixed value dtypes
     srv.drain()
+
+
+def test_rows_of_one_vector(arrow, pool):
+    """Requests of 16-byte rows (k = 8): their permute-out is a pass of its own, after the last of an
+    odd or even number of iterations, alone and beside wider requests."""
+    mats, hs = pool
+    gen = torch.Generator(device="cuda").manual_seed(6)
+    for ks in ((8, 8, 8, 8), (8, 64, 8, 16)):
+        srv = arrow.ArrowServer(hbm_budget=1 << 28, max_active=8, x_dtype="bf16")
+        runs = []
+        for m, k in enumerate(ks):
+            for it in (0, 1, 2, 5):
+                X = torch.randn(mats[m].n, k, device="cuda", generator=gen).bfloat16()
+                Y = torch.full_like(X, float("nan"))
+                srv.submit(hs[m], X, Y, it)
+                runs.append((m, X, Y, it))
+            srv.step()
+        srv.drain()
+        assert srv.stats()["status"] == 0
+        for m, X, Y, it in runs:
+            assert torch.equal(Y, hs[m].spmm(X, it)), (m, it)
+        srv.close()
