@@ -1115,7 +1115,16 @@ static int make_plan(const arrow_handle_s* h, int64_t k, int x_dtype, int flags,
     const int64_t n_tiles = h->tile_row.empty() ? 0 : int64_t(h->tile_row.size()) - 1;
     const int cap = (flags & ARROW_RESCALE) ? ARROW_ROWS_MIN_BLOCKS_RESCALE : ARROW_ROWS_MIN_BLOCKS;
     const int64_t most = int64_t(sm) * std::min(h->tune.ctas_per_sm, cap);
-    p.parts = share ? row_parts(n_tiles, most, h->tune.tile_rows, 256 / p.T) : 1;
+    // With the rescale every CTA also ends with FP64 sums of its columns (about two FP64 operations per clock
+    // and SM), which more CTAs repeat: narrow rows share tiles up to one CTA per SM only, wide ones
+    // (whose rows are longer chains and whose sums take fewer steps) up to two, or three where that
+    // gives every tile two.  10 iterations in us, up to all resident CTAs / no sharing / this rule: 150^2
+    // grid (88 tiles) k = 32 BF16 168 / 118 / 118, k = 128 BF16 233 / 178 / 158; 250 x 200 grid (196 tiles)
+    // k = 128 FP32 276 / 264 / 219.
+    int64_t share_most = most;
+    if (flags & ARROW_RESCALE)
+        share_most = std::min<int64_t>(most, p.T < 16 ? sm : std::max<int64_t>(2 * sm, std::min<int64_t>(3 * sm, 2 * n_tiles)));
+    p.parts = share ? row_parts(n_tiles, share_most, h->tune.tile_rows, 256 / p.T) : 1;
     p.rows_grid = int(std::max<int64_t>(1, std::min<int64_t>(n_tiles * p.parts, most)));
     const int64_t n_long = int64_t(h->long_rows.size());
     const int64_t teams = 256 / p.T;

@@ -128,3 +128,21 @@ def test_x_and_y_overlap_in_part(arrow, fold_in, shift):
         M.spmm(X, iters, out=Y)
         torch.cuda.synchronize()
         assert torch.equal(Y, ref)
+
+
+@pytest.mark.parametrize("dims", [(40, 37), (150, 150), (250, 200), (300, 290)])
+@pytest.mark.parametrize("dt,k", [("f32", 8), ("f32", 64), ("f32", 256), ("bf16", 128)])
+def test_rescale_with_shared_tiles(arrow, dims, dt, k):
+    """The column rescale where tiles are shared by several CTAs, by two and by none (6 to 340 tiles),
+    narrow and wide rows, against the FP64 oracle (FP32 1e-5 per iteration, BF16 2e-2 in the 2-norm)."""
+    A = w.grid_stencil(dims, seed=8)
+    M = arrow.ArrowMatrix(A, 64, value_dtype=dt)
+    X = torch.from_numpy(w.features(A.n, k, seed=9)).to("cuda", {"f32": torch.float32, "bf16": torch.bfloat16}[dt])
+    Y = M.spmm(X, 3, rescale=True)
+    assert torch.equal(Y, M.spmm(X, 3, rescale=True)) and M.status() == 0
+    Y = Y.float().cpu().numpy().astype(np.float64)
+    R = S.iterate(A, X.float().cpu().numpy().astype(np.float64), 3, rescale=True)
+    if dt == "f32":
+        assert np.max(np.max(np.abs(Y - R), axis=0) / np.max(np.abs(R), axis=0)) <= 1e-5 * 3
+    else:
+        assert np.max(np.linalg.norm(Y - R, axis=0) / np.linalg.norm(R, axis=0)) <= 2e-2
