@@ -128,6 +128,7 @@ struct arrow_handle_s {
     double decompose_seconds = 0.0;
     bool uploaded = false;
     bool long_desc = true;   // some short row has more entries than its descriptor holds (kLongDesc)
+    bool even_rows = false;  // short rows of nearly one length: mean square at most 1.2 times the squared mean
     // bumped whenever the device arrays or the tile table change (upload, re-tiling):
     // batches that cached descriptors or work-unit counts of this handle rebuild them
     uint64_t generation = 0;

@@ -146,3 +146,25 @@ def test_rescale_with_shared_tiles(arrow, dims, dt, k):
         assert np.max(np.max(np.abs(Y - R), axis=0) / np.max(np.abs(R), axis=0)) <= 1e-5 * 3
     else:
         assert np.max(np.linalg.norm(Y - R, axis=0) / np.linalg.norm(R, axis=0)) <= 2e-2
+
+
+@pytest.mark.parametrize("case", ["even", "uneven", "long"])
+@pytest.mark.parametrize("dt,k", [("f32", 128), ("f32", 384), ("bf16", 256)])
+def test_wide_rows_in_row_order(arrow, case, dt, k):
+    """Rows of 32 vectors come in row order where the lengths are even (one length, or 100 to 140: longer than
+    a descriptor holds) and by length where they are not: the bits of narrower calls on slices of
+    the columns, which always come by length."""
+    n = 2049
+    rng = np.random.default_rng(15)
+    A = {"even": lambda: w.rgg(n, seed=16), "uneven": lambda: _matrix(n),
+         "long": lambda: _matrix_of(rng.integers(100, 141, n), 17)}[case]()
+    ln = np.diff(A.rowptr).astype(np.float64)
+    assert ((ln ** 2).mean() <= 1.2 * ln.mean() ** 2) == (case != "uneven")
+    M = arrow.ArrowMatrix(A, 64, value_dtype=dt, long_row=256)
+    X = torch.from_numpy(w.features(n, k, seed=18)).to("cuda", {"f32": torch.float32, "bf16": torch.bfloat16}[dt])
+    for tile in ((256, 2048), (2048, 8192), (32, 1024)):
+        M.set_tuning(tile[0], tile[1], 2, 70)
+        Y = M.spmm(X, 2)
+        for c in range(0, k, 64):
+            assert torch.equal(Y[:, c:c + 64], M.spmm(X[:, c:c + 64].contiguous(), 2))
+    assert M.status() == 0
