@@ -112,7 +112,9 @@ void launch_step(arrow_server_s* S, const int64_t* tot, int n_m, cudaStream_t s)
     const int ctas = S->active.empty() ? 3 : std::min(S->active[0].h->tune.ctas_per_sm, kBatchMinBlocks);
     const int carve = S->active.empty() ? 75 : S->active[0].h->tune.carveout;
     const int sm = S->sm_count;
-    const int parts = row_parts(tot[2], int64_t(sm) * ctas, rows_max, 32);
+    bool narrow = true;   // every request's rows are one vector
+    for (const auto& r : S->active) narrow = narrow && r.k * int64_t(sizeof(TX)) == 16;
+    const int parts = narrow ? 1 : row_parts(tot[2], int64_t(sm) * ctas, rows_max, 32);
     auto args = [&](int cls, int parity, int dir) {
         return BatchArgs{S->d_desc, db + cls * (n_m + 1), n_m, tot[cls], parity, dir, 0, S->d_status, L.rp, L.col, L.buf, parts};
     };
@@ -126,7 +128,7 @@ void launch_step(arrow_server_s* S, const int64_t* tot, int n_m, cudaStream_t s)
            grid_w(tot[1], 8), 256, 0, args(1, 0, 0));
     if (tot[2]) {
         const int g = int(std::max<int64_t>(1, std::min<int64_t>(tot[2] * parts, int64_t(sm) * ctas)));
-        go(arrow_batch_rows_kernel<TX, TV>, g, 256, batch_smem_bytes(L), args(2, 0, 0));
+        go(narrow ? arrow_batch_rows_kernel<TX, TV, true> : arrow_batch_rows_kernel<TX, TV, false>, g, 256, batch_smem_bytes(L), args(2, 0, 0));
     }
     if (tot[3]) go(arrow_batch_combine_kernel<TX>, grid_w(tot[3], 4), 256, 0, args(3, 0, 0));
     if (tot[4]) go(arrow_batch_gather_kernel<TX>, grid_w(tot[4], 8), 256, 0, args(4, 1, 1));

@@ -432,6 +432,22 @@ __device__ __forceinline__ void gather_row(const int32_t* scol, const TV* sval, 
     }
 }
 
+// The same sum in rounds of 8 whose slots past the row's end are predicated off: one code path for all
+// the teams of a warp, whatever their row lengths.
+template <typename TX, typename TV>
+__device__ __forceinline__ void gather_row_pred(const int32_t* scol, const TV* sval, int s, int e, const TX* X,
+                                                int64_t ldx, float* acc) {
+    for (int base = s; base < e; base += 8) {
+        uint4 x[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (u < e - base) x[u] = ld_x(X + int64_t(scol[base + u]) * ldx);
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (u < e - base) axpy_vec<TX, TV>(sval[base + u], x[u], acc);
+    }
+}
+
 // Row descriptors: one 32-bit word per row, every tile's rows in order of decreasing length
 // (equal lengths in row order), so that the teams of a warp walk rows of the same length
 // together.  In row order the exact remainder rounds of gather_row diverge on every warp whose

@@ -168,3 +168,28 @@ def test_member_retiled_with_nothing_else_changed(arrow):
             torch.cuda.synchronize()
             assert B.status() == 0
             assert all(torch.equal(y, r) for y, r in zip(Ys, ref))
+
+
+@pytest.mark.parametrize("dt,k", [("f32", 4), ("bf16", 8)])
+def test_batch_of_rows_of_one_vector(arrow, dt, k):
+    # every member's rows are one vector: rows of 0 to 140 entries in row order and predicated rounds, tiles of
+    # 32 to 2048 rows, against the single calls (rows by length, exact rounds)
+    tdt = {"f32": torch.float32, "bf16": torch.bfloat16}[dt]
+    rng = np.random.default_rng(31)
+    counts = rng.choice(np.array([0, 1, 7, 8, 9, 16, 17, 63, 64, 140]), 2049)
+    rowptr = np.concatenate([[0], np.cumsum(counts)])
+    col = np.concatenate([np.sort(rng.choice(2049, c, replace=False)) for c in counts]).astype(np.int32)
+    mats = [w.Csr(2049, rowptr, col, rng.uniform(0.5, 1.5, col.size)), w.rgg(1500, seed=32), w.grid_stencil((7, 5), seed=33),
+            w.rmat_gcn(9, 16, seed=34)]
+    ms = [arrow.ArrowMatrix(A, 32, value_dtype=dt, long_row=256 if A.n == 2049 else 32) for A in mats]
+    Xs = [torch.from_numpy(w.features(A.n, k, seed=i)).to("cuda", tdt) for i, A in enumerate(mats)]
+    B = arrow.ArrowBatch(ms)
+    for tile in ((256, 2048), (2048, 8192), (32, 1024)):
+        for M in ms:
+            M.set_tuning(tile[0], tile[1], 2, 70)
+        for it in (1, 4):
+            ref = [M.spmm(X, it) for M, X in zip(ms, Xs)]
+            for graph in (False, True):
+                for y, r in zip(B.spmm(Xs, it, graph=graph), ref):
+                    assert torch.equal(y, r)
+    assert B.status() == 0
