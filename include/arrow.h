@@ -96,8 +96,8 @@ int arrow_opts_default(arrow_opts* o);
  * through a second copy of the column indices in vertex ids (4 bytes per entry of device
  * memory, set up when the setting is applied) instead of permuting X into pi_0 order first.
  * fused_small = 1 runs a whole arrow_spmm call as one cooperative launch (permute-in, every
- * iteration's phases separated by grid-wide barriers with a 2 s limit, permute-out) when the
- * problem is small (n <= 2^20, nnz <= 2^23) and k / (16 / sizeof(x_dtype)) <= 32, where kernel
+ * iteration's phases separated by grid-wide barriers with a 2 s limit, with ARROW_RESCALE the
+ * permute-out) when the problem is small (n <= 2^20, nnz <= 2^23) and k / (16 / sizeof(x_dtype)) <= 32, where kernel
  * start-up would dominate; identical results without ARROW_RESCALE, within rounding with it
  * (the FP64 column sums are grouped differently).  Larger problems ignore it.
  * Defaults: 256, 2048, 4, 70, 0, 0. */
@@ -183,8 +183,9 @@ void arrow_free(arrow_handle h);
  * X is permuted into the first level's order once, every step runs the split head-row
  * reduction and the fused arrow-row kernel (all levels, fixed level order, no atomics),
  * and the result is permuted back once (Section 5.1: rows stay in pi_0 order between
- * iterations): by the last iteration's stores, or with ARROW_RESCALE in a pass of its own.  sigma (Section 2 leaves it to the application) is composed from three
- * optional parts in a fixed order, sigma(Y) = colnorm(rownorm(relu(Y))):
+ * iterations): by the last iteration's stores, or with ARROW_RESCALE or rows under 32 bytes in a pass
+ * of its own.  sigma (Section 2 leaves it to the application) is composed from three optional
+ * parts in a fixed order, sigma(Y) = colnorm(rownorm(relu(Y))):
  *   ARROW_RELU    -- max(0, y) on every element (the non-linearity of a graph-network
  *                    layer, the use the introduction motivates), fused into the row store;
  *   ARROW_ROWNORM -- every row divided by its L2 norm (zero rows stay zero), fused into the
@@ -256,8 +257,9 @@ int arrow_batch_create(const arrow_handle* handles, int32_t count, arrow_batch* 
  * X[m], Y[m] DEVICE pointers (host arrays of count pointers), row-major n_m x k[m], 16-byte
  * aligned, element type x_dtype; k[m] = V * 2^j with V = 16 / sizeof(x_dtype) and k[m] / V <= 32.
  * Each iteration of the whole batch is one launch per kernel class (split-row segments,
- * rows, split-row combine) over the work units of all matrices; the permutes are one launch
- * each.  Results are bit-identical to arrow_spmm on each matrix alone.  flags: 0 or
+ * rows, split-row combine) over the work units of all matrices; the permute-in is one launch,
+ * and so is the permute-out of the members with rows under 32 bytes (the others' last iteration
+ * stores into Y).  Results are bit-identical to arrow_spmm on each matrix alone.  flags: 0 or
  * ARROW_GRAPH (capture once, replay while X, Y, k, iters and dtype stay the same).  The call
  * allocates its workspace on first use or growth (outside any capture) and synchronises
  * the stream when X, Y, k or dtype change.  The batch's device must be current (ARROW_EINVAL
@@ -314,7 +316,8 @@ int arrow_server_submit(arrow_server s, arrow_handle h, const void* X, void* Y, 
 
 /* One step: retire requests the GPU has finished, admit queued requests in arrival order
  * while a slot and budget are free, launch one iteration of every active request (plus the
- * permute-in of new ones and the permute-out of finishing ones) on `stream`, which must be
+ * permute-in of new ones; a last iteration stores into its Y, rows under 32 bytes and requests of
+ * no iteration by a permute-out) on `stream`, which must be
  * the same for every step.  Waits for the oldest step only when max_inflight steps are queued.
  * The server's device must be current (ARROW_EINVAL otherwise, nothing launched).
  * *active receives the number of active requests (may be NULL).  Errors: ARROW_EINVAL, ARROW_ECUDA. */

@@ -46,8 +46,8 @@ int require_device(int device, const char* what);
 void set_smem_attrs(const void* fn, int carveout, bool dynamic);
 
 // Row tiles of the fused row program: by default at most kTileRows rows and kTileNnz entries
-// each (arrow_set_tuning / arrow_autotune change them per handle).  A tile's row pointers and
-// entries are staged into shared memory with bulk copies.
+// each (arrow_set_tuning / arrow_autotune change them per handle).  A tile's row descriptors
+// and entries are staged into shared memory with bulk copies.
 #ifndef ARROW_TILE_NNZ
 #define ARROW_TILE_NNZ 2048
 #endif

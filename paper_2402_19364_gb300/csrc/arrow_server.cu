@@ -128,7 +128,8 @@ void launch_step(arrow_server_s* S, const int64_t* tot, int n_m, cudaStream_t s)
            grid_w(tot[1], 8), 256, 0, args(1, 0, 0));
     if (tot[2]) {
         const int g = int(std::max<int64_t>(1, std::min<int64_t>(tot[2] * parts, int64_t(sm) * ctas)));
-        go(narrow ? arrow_batch_rows_kernel<TX, TV, true> : arrow_batch_rows_kernel<TX, TV, false>, g, 256, batch_smem_bytes(L), args(2, 0, 0));
+        go(narrow ? arrow_batch_rows_kernel<TX, TV, true> : arrow_batch_rows_kernel<TX, TV, false>, g, 256,
+           batch_smem_bytes(L), args(2, 0, 0));
     }
     if (tot[3]) go(arrow_batch_combine_kernel<TX>, grid_w(tot[3], 4), 256, 0, args(3, 0, 0));
     if (tot[4]) go(arrow_batch_gather_kernel<TX>, grid_w(tot[4], 8), 256, 0, args(4, 1, 1));

@@ -135,7 +135,7 @@ __device__ __forceinline__ void flush_squares(float* sq, double* slot, int lane)
     }
 }
 
-// Thread 0: stage tile t (row pointers, columns, values) into buf with three bulk copies.
+// Thread 0: stage tile t (row descriptors or pointers, columns, values) into buf with three bulk copies.
 template <typename TV>
 __device__ __forceinline__ void issue_tile(const RowArgs& a, int t, unsigned char* buf, uint64_t* bar) {
     stage_tile<TV>(a.row_desc, a.col, static_cast<const TV*>(a.val), a.tile_row[t], a.tile_row[t + 1], a.tile_ent[t],
@@ -143,7 +143,7 @@ __device__ __forceinline__ void issue_tile(const RowArgs& a, int t, unsigned cha
 }
 
 // Fused arrow-row kernel (persistent).  Each CTA walks row tiles t = blockIdx.x, +gridDim.x,
-// ...; a tile's row pointers and entries arrive by bulk copy into one of kStages buffers.
+// ...; a tile's row descriptors and entries arrive by bulk copy into one of kStages buffers.
 // Warps are not synchronised per tile: every warp takes its rows of the tile as soon as the
 // tile has landed, and the last warp done with a buffer re-arms it with the tile kStages
 // ahead.  A team of T lanes owns a row: it reads up to 8 entries from shared memory, issues
@@ -608,8 +608,8 @@ struct FusedArgs {
 // The whole arrow_spmm call in one cooperative launch, for problems small enough that kernel
 // start-up dominates: the permute-in, then per iteration the split-row segments and the rows
 // (one phase), the combine of the split rows, and the FP64 column sums (every CTA sums the
-// per-CTA partials itself, in the same order), then the permute-out.  Each row and segment is
-// computed with the same code and order as the multi-launch path (identical bits without the
+// per-CTA partials itself, in the same order), then the permute-out (without the rescale the last
+// iteration stores its rows at their vertices instead).  Each row and segment is computed with the same code and order as the multi-launch path (identical bits without the
 // rescale; with it the column sums are grouped by this launch's CTAs).  Needs k / V <= 32 (one
 // chunk).  A barrier that runs out sets the status word and the kernel returns.
 // Bound by latency: per iteration one row per team (dependent loads of its entries and X rows from
@@ -1314,7 +1314,9 @@ static int launch_fused(const arrow_handle_s* h, const Plan& p, const void* X, i
 // Whether the last iteration stores its rows straight into the caller's Y (row p at vertex
 // pi_0^{-1}(p)) instead of a permute-out reading and writing them once more.  Not with the column
 // rescale, whose last factors are known only after the last row.  Not for rows of less than a
-// 32-byte sector, which scattered stores would write in halves.  And not when the same launch
+// 32-byte sector, of which a scattered store writes half; measured, the pass costs more there too
+// (pass / stores: 160^3 grid, k = 4 FP32, one product 160 / 126 us, 10 iterations 826 / 791;
+// random-geometric 100,003 rows 71 / 66), so this line is only where it was first drawn.  And not when the same launch
 // reads the caller's X (one iteration with the permute-in folded in) and X and Y overlap.
 static bool fold_permute_out(const arrow_handle_s* h, const void* X, const void* Y, int64_t k, int sx, int iters, int flags,
                              bool folded_in) {

@@ -59,8 +59,8 @@ __device__ __forceinline__ int find_mat(const int64_t* base, int n, int64_t w) {
 }
 
 // The last iteration of a matrix stores its rows straight at their vertices in the caller's Y
-// (row p at pi_0^{-1}(p)), without a permute-out pass; rows narrower than a 32-byte sector keep
-// the pass, which would be written in halves.
+// (row p at pi_0^{-1}(p)), without a permute-out pass; rows narrower than a 32-byte sector keep the pass
+// (fold_permute_out, arrow_spmm.cu, has the reason and the figures).
 __host__ __device__ inline bool folds_out(int64_t k, int sx) { return k * sx >= 32; }
 
 inline int batch_smem_bytes(const TileLayout& L) { return 128 + kStages * L.buf; }

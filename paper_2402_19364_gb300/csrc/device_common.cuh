@@ -143,9 +143,9 @@ __device__ __forceinline__ void axpy_vec<float, float>(float w, const uint4& x, 
 // visible.  Every thread of every kernel waits before it reads or writes anything that changes
 // during a call, and lets the next kernel start only after that (pdl_launch(), or its end), so at
 // most two kernels overlap and a kernel's completion implies that of all before it.
-// What it takes off a launch: 64 x 64 grid, 10 iterations 67.6 -> 48.4 us per call; 100^3 grid, 20
-// iterations with the rescale 1174 -> 1067; R-MAT 16 FP32, 3 iterations 184 -> 161; 24-matrix FP16
-// batch 1974 -> 1960.  The gather, segment, combine and norm kernels let the next start
+// What it takes off a launch, alone: 64 x 64 grid, 10 iterations 67.6 -> 48.4 us per call (44.5 with one
+// shared-memory split, below); 100^3 grid, 20 iterations with the rescale 1174 -> 1067; R-MAT 16 FP32,
+// 3 iterations 184 -> 161; 24-matrix FP16 batch 1974 -> 1960.  The gather, segment, combine and norm kernels let the next start
 // at their end only: a rows kernel that came in while a permute was running cost 8 us (BF16 layer
 // 61.5 -> 69.5 us) and R-MAT 16 went from 161 to 178.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
@@ -349,8 +349,8 @@ __device__ __forceinline__ void segment_partial(const int32_t* __restrict__ col,
 
 // segment_partial where a launch has few segments: the same entries in the same order (the same bits),
 // 16 gathers in flight instead of 8 and the next 16 columns and values loaded while they fly, so a
-// long segment is a chain of a quarter as many memory latencies.  It takes about 150 registers (8
-// warps per SM), so it is used where those warps take at most one segment each (seg_ahead): R-MAT
+// long segment is a chain of a quarter as many memory latencies.  It takes about 150 registers (230
+// in the batched kernel, which holds every width; 8 warps per SM either way), so it is used where those warps take at most one segment each (seg_ahead): R-MAT
 // 13, 892 segments, 10 iterations 290 -> 260 us per call at k = 128 BF16 and 162 -> 150 at k = 16
 // FP32, 299 -> 268 on the one-launch path (which has one CTA per SM and always takes it); with
 // 2,374 segments it lost, 346 -> 387.
@@ -454,9 +454,10 @@ __device__ __forceinline__ void gather_row_pred(const int32_t* scol, const TV* s
 // rows differ: a random-geometric warp of 8 teams ran up to 7 remainder sizes one after the
 // other, each with its own memory latency (random-geometric graph, 1 M rows, k = 32 FP16: 96
 // -> 63 us per product; R-MAT 20, k = 128 BF16: 1.09x on the whole call; grids, whose rows are
-// all alike, within 1 %: 256^3 grid rows kernel 0.650 -> 0.643 ms by the end).  Fields: first entry within the tile (15 bits: a
-// tile has at most 16384 entries), row within the tile (11 bits: at most 2048 rows), length (6
-// bits; kLongDesc means "kLongDesc or more", read from the row pointers).  They take the place of
+// all alike, within 1 %: 256^3 grid rows kernel 0.650 -> 0.643 ms by the end).  Where a warp has one row at a time
+// (rows_in_order, arrow_spmm.cu) or 32 (the batched kernel's NARROW form) the row pointers are staged
+// instead.  Fields: first entry within the tile (15 bits: a tile has at most 16384 entries), row
+// within the tile (11 bits: at most 2048 rows), length (6 bits; kLongDesc means "kLongDesc or more", read from the row pointers).  They take the place of
 // the row pointers in the staged tile: the same bytes.
 constexpr uint32_t kLongDesc = 63;
 __host__ __device__ inline uint32_t row_desc_pack(uint32_t start, uint32_t row, uint32_t len) {
@@ -507,9 +508,9 @@ __device__ __forceinline__ void drain_pipeline(PipeSmem* ps) {
 }
 
 // Shared-memory layout of one staged tile of at most tile_rows rows and tile_nnz entries: row
-// pointers, column indices and values, each a 16-byte aligned superset of the tile's range.
+// descriptors (or pointers), column indices and values, each a 16-byte aligned superset of the tile's range.
 struct TileLayout {
-    int rp, col, buf;   // bytes of the row-pointer and column regions, bytes of one whole buffer
+    int rp, col, buf;   // bytes of the row-descriptor and column regions, bytes of one whole buffer
 };
 __host__ __device__ inline TileLayout tile_layout(int tile_rows, int tile_nnz) {
     TileLayout L;
@@ -522,7 +523,8 @@ __host__ __device__ inline TileLayout tile_layout(int tile_rows, int tile_nnz) {
 // CTAs that share the rows of one tile.  Fewer tiles than resident CTAs (`most`) leave SMs idle while
 // every team walks several rows, each a chain of dependent loads: then as many CTAs as there is
 // room for stage the same tile, and each takes every parts-th group of rows, down to one row per
-// team.  64 x 64 grid (16 tiles, 4 rows per team), 10 iterations: 44.5 -> 36 us per call.
+// team.  64 x 64 grid (16 tiles, 4 rows per team), 10 iterations: 44.5 -> 36 us per call.  (With the column
+// rescale fewer: make_plan.)
 inline int row_parts(int64_t n_tiles, int64_t most, int tile_rows, int teams) {
     if (n_tiles <= 0) return 1;
     const int64_t useful = (tile_rows + teams - 1) / teams;
