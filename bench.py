@@ -11,10 +11,13 @@ Inputs (X 4.1 GB, A 3.6 GB) are larger than the 129 MB L2, so no flush is needed
                   [--workload grid3d|grid2d|rmat|batch|serve|predicates] [--size S] [--iters T] [--k K]
                   [--dtype f32|bf16] [--count M] [--tuning R,E,C,P] [--no-e2e] [--no-cpu] [--no-cusparse]
 
-The line carries the device-timed value, the rows kernel's roofline, per-step min/mean/max,
+The record holds the device-timed value, the rows kernel's roofline, per-step min/mean/max,
 the clocks seen during the timed region, an end-to-end figure through the public call with
 pinned host buffers (copies inside the timed region; two steps in flight on two streams,
-and the one-stream form beside it), cuSPARSE on the undecomposed matrix and the CPU oracle.
+and the one-stream form beside it), cuSPARSE on the undecomposed matrix, the CPU oracle and, in the
+default run, the other configurations.  The line on standard output is its short form
+(short_line: a run's output may be kept from its end only); the whole record goes to standard
+error, or with --full is the line.
 The rows kernel is autotuned before timing unless --tuning fixes its launch configuration.
 --impl reference times the CPU oracle (the FP64 product of the oracle package, as it
 stands) on a bounded sample of the same workload on the host cores.
@@ -61,6 +64,7 @@ def parse():
     p.add_argument("--no-device-decompose", action="store_true",
                    help="skip timing the decomposition with its steps on the GPU")
     p.add_argument("--no-sub", action="store_true", help="default workload only: skip the other configurations' records")
+    p.add_argument("--full", action="store_true", help="print the whole record as the line")
     p.add_argument("--sub", default="grid2d,rmat,batch,serve,predicates", help="which other configurations to attach")
     p.add_argument("--tuning", default="", help="tile_rows,tile_nnz,ctas_per_sm,carveout[,fold_permute_in[,fused_small]]: fixed tuning "
                    "instead of autotuning (keeps a profiler's launch list short)")
@@ -739,6 +743,37 @@ def cusparse_record(A, M, Xd, spec, dt_name, stream, reps=5):
     return rec
 
 
+def short_line(out):
+    """The headline's keys of a record and one figure of each other configuration, within 1,400
+    characters: a line longer than the end of the output that a caller keeps cannot be read."""
+    def num(v):
+        return float(f"{v:.6g}") if isinstance(v, float) else v
+
+    def pick(d, *keys):
+        return {k: num(d[k]) for k in keys if k in d}
+
+    line = pick(out, "metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+                "vs_baseline", "dtype", "data", "gpu_launches")
+    line["config"] = pick(out["config"], "workload", "b", "k", "iters", "parallelism")
+    line["config"]["l2"] = out["config"]["l2"].split(":")[0]
+    line["roofline"] = pick(out["roofline"], "bound", "achieved", "peak", "unit", "frac", "traffic")
+    line["clocks"] = pick(out["clocks"], "sm_mhz", "sm_max_mhz", "reasons")
+    if "e2e" in out:
+        line["e2e"] = pick(out["e2e"], "value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step")
+    if "us_per_iter" in out:
+        line["us_per_iter"] = num(out["us_per_iter"])
+    if "cusparse" in out:
+        line["cusparse_iters_per_s"] = num(out["cusparse"].get("iters_per_s"))
+    if "cpu_baseline" in out:
+        line["cpu_baseline"] = pick(out["cpu_baseline"], "value", "unit", "cores", "kind")
+    sub = out.get("configs", {})
+    figures = {"grid2d": ("us_per_iter",), "rmat": ("value",), "batch": ("value", "speedup_vs_fp32"),
+               "serve": ("value", "p50_ms", "p99_ms")}
+    if sub:
+        line["configs"] = {c: pick(sub[c], *keys) for c, keys in figures.items() if c in sub}
+    return line
+
+
 # Configurations measured beside the headline in the default run (each in its own process,
 # after the headline's device memory is released): (key, bench arguments).
 SUBRECORDS = [
@@ -758,7 +793,7 @@ def run_subrecords(keys, timeout_s=1800):
             continue
         t0 = time.perf_counter()
         try:
-            r = subprocess.run([sys.executable, os.path.abspath(__file__), *args], cwd=ROOT, capture_output=True,
+            r = subprocess.run([sys.executable, os.path.abspath(__file__), "--full", *args], cwd=ROOT, capture_output=True,
                                text=True, timeout=timeout_s)
             lines = [ln for ln in r.stdout.splitlines() if ln.startswith("{")]
             if r.returncode != 0 or not lines:
@@ -1020,7 +1055,9 @@ def main():
         torch.cuda.empty_cache()
         out["configs"] = run_subrecords([x for x in a.sub.split(",") if x])
     if rank == 0:
-        print(json.dumps(out), flush=True)
+        if not a.full:
+            print("record: " + json.dumps(out), file=sys.stderr, flush=True)
+        print(json.dumps(out if a.full else short_line(out)), flush=True)
     if pg is not None:
         pg.destroy_process_group()
 

@@ -122,3 +122,43 @@ def test_every_default_subrecord_is_a_known_workload():
         wl = args[args.index("--workload") + 1]
         assert wl in ("grid2d", "rmat", "batch", "serve", "predicates"), (key, wl)
     assert [k for k, _ in bench.SUBRECORDS] == ["grid2d", "rmat", "batch", "serve", "predicates"]
+
+
+def test_short_line_fits_and_keeps_the_contract():
+    """The line that a caller parses from the end of the output: every key of the headline, at most
+    1,400 characters with the longest values a run gives."""
+    import json
+    x = 123456.789012345678
+    spec = bench.workload_spec(_args())
+    out = {"metric": bench.METRIC, "value": x, "unit": "iters/s", "n_gpus": 1, "steps": 100, "warmup": 10,
+           "ms_per_step": x, "step_ms": {"mean": x}, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
+           "dtype": "bf16", "data": "synthetic",
+           "config": {"workload": max((bench.workload_spec(_args(workload=v))["desc"] for v in ("grid3d", "grid2d", "rmat")),
+                                      key=len),
+                      "n": spec["N"] ** 3, "b": 4096, "k": 128, "iters": 20, "levels": [[64000000, 353300000]] * 20,
+                      "l2": "inputs smaller than L2: a 512 MiB buffer is written", "parallelism": "replicas x1"},
+           "roofline": {"bound": "hbm", "achieved": x, "peak": 6784.2, "unit": "GB/s", "frac": x, "traffic": 13361697894.0,
+                        "peak_kind": "measured"},
+           "gpu_launches": 123456, "clocks": {"sm_mhz": 2070.0, "sm_max_mhz": 2070.0, "reasons": ["sw_power_cap", "gpu_idle"],
+                                              "samples": 1000},
+           "e2e": {"value": x, "unit": "iters/s", "h2d_bytes_per_step": 4096000000, "d2h_bytes_per_step": 4096000000,
+                   "ms_per_step": x, "one_stream": {"value": x}},
+           "cusparse": {"iters_per_s": x, "variants": [x] * 100}, "us_per_iter": x,
+           "cpu_baseline": {"value": x, "unit": "iters/s", "cores": 16, "kind": "oracle", "sample": "..."},
+           "configs": {"grid2d": {"us_per_iter": x}, "rmat": {"value": x, "config": {}},
+                       "batch": {"value": x, "speedup_vs_fp32": x}, "serve": {"value": x, "p50_ms": x, "p99_ms": x},
+                       "predicates": {"cases": []}}}
+    line = bench.short_line(out)
+    text = json.dumps(line)
+    assert len(text) <= 1400 and "\n" not in text
+    for key in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+                "vs_baseline", "dtype", "data", "config", "e2e", "gpu_launches", "clocks"):
+        assert key in line
+    assert set(line["e2e"]) == {"value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step"}
+    assert set(line["clocks"]) == {"sm_mhz", "sm_max_mhz", "reasons"}
+    assert abs(line["value"] / x - 1) < 1e-5 and line["steps"] == 100
+    # a record without the optional parts, or with a failed configuration, has a line too
+    for key in ("e2e", "cusparse", "cpu_baseline", "us_per_iter"):
+        del out[key]
+    out["configs"] = {"rmat": {"error": "rc=1", "wall_s": x}}
+    assert bench.short_line(out)["configs"] == {"rmat": {}}
