@@ -68,7 +68,7 @@ static inline int rows_smem_bytes(const TileLayout& L, int norm_doubles) { retur
 
 struct RowArgs {
     const int32_t* long_rowptr;   // row pointers, for rows of kLongDesc entries or more; null if there are none
-    const uint32_t* row_desc;     // or (in_order) the row pointers
+    const uint32_t* row_desc;     // or (IN_ORDER) the row pointers
     const int32_t* col;
     const void* val;
     const int32_t* tile_row;
@@ -86,7 +86,6 @@ struct RowArgs {
     const int32_t* out_idx;    // row r is stored at row out_idx[r] of Y (permute-out folded in), or null
     int32_t rp_bytes, col_bytes, buf_bytes;   // shared-memory layout of a staged tile
     int32_t sigma;             // kSigmaRelu | kSigmaRowNorm applied to each output row, or 0
-    int32_t in_order;          // T = 32: the rows of a tile in row order (rows_in_order)
 };
 
 // sigma applied to an output row held by a team of T lanes (V columns each) before it is
@@ -148,8 +147,9 @@ __device__ __forceinline__ void issue_tile(const RowArgs& a, int t, unsigned cha
 // tile has landed, and the last warp done with a buffer re-arms it with the tile kStages
 // ahead.  A team of T lanes owns a row: it reads up to 8 entries from shared memory, issues
 // their 16-byte X gathers together, accumulates in FP32 in entry order (levels in order),
-// scales, stores the row and, with RESCALE, adds its squares to FP64 per-column sums.
-template <typename TX, typename TV, int T, bool RESCALE>
+// scales, stores the row and, with RESCALE, adds its squares to FP64 per-column sums.  IN_ORDER: a tile's
+// rows in row order, from the row pointers (rows_in_order).
+template <typename TX, typename TV, int T, bool RESCALE, bool IN_ORDER>
 __global__ void __launch_bounds__(256, RESCALE ? ARROW_ROWS_MIN_BLOCKS_RESCALE : ARROW_ROWS_MIN_BLOCKS)
     arrow_rows_kernel(RowArgs a) {
     using P = Pack<TX>;
@@ -217,8 +217,8 @@ __global__ void __launch_bounds__(256, RESCALE ? ARROW_ROWS_MIN_BLOCKS_RESCALE :
         const int step = TEAMS * a.parts;
         uint32_t dn = sdesc[min(q0, nrows)];
         for (int q = q0; q < nrows; q += step) {
-            const RowDesc rd = T == 32 && a.in_order ? RowDesc{int(dn) - e0, q, int(sdesc[q + 1] - dn)}
-                                                     : row_desc_unpack(dn, a.long_rowptr, r0);
+            const RowDesc rd = IN_ORDER ? RowDesc{int(dn) - e0, q, int(sdesc[q + 1] - dn)}
+                                        : row_desc_unpack(dn, a.long_rowptr, r0);
             dn = sdesc[min(q + step, nrows)];
             const int s = rd.start, e = rd.start + rd.len;
             // (with the rescale the permute-out is never folded in)
@@ -1207,14 +1207,13 @@ static void launch_step(const arrow_handle_s* h, const Plan& p, const TX* cur, T
         const bool in_order = rows_in_order(h, p);
         RowArgs ra{h->long_desc ? d.rowptr : nullptr, in_order ? reinterpret_cast<const uint32_t*>(d.rowptr) : d.row_desc, col,
                    d.val, d.tile_row, d.tile_ent, n_tiles, p.parts, cur, nxt, k, koff, p.kc, scale_in, np, d.status, out_idx,
-                   L.rp, L.col, L.buf, sigma, in_order};
+                   L.rp, L.col, L.buf, sigma};
         const int smem = rows_smem_bytes(L, np ? 8 * p.kc : 0);
         cudaEvent_t e0 = pf.begin();
-        if (np) {
-            go(arrow_rows_kernel<TX, TV, T, true>, p.rows_grid, 256, smem, ra);
-        } else {
-            go(arrow_rows_kernel<TX, TV, T, false>, p.rows_grid, 256, smem, ra);
-        }
+        auto rows = np ? arrow_rows_kernel<TX, TV, T, true, false> : arrow_rows_kernel<TX, TV, T, false, false>;
+        if constexpr (T == 32)
+            if (in_order) rows = np ? arrow_rows_kernel<TX, TV, T, true, true> : arrow_rows_kernel<TX, TV, T, false, true>;
+        go(rows, p.rows_grid, 256, smem, ra);
         pf.end(ARROW_K_ROWS, e0);
         if (p.comb_grid) {
             CombArgs ca{d.long_rows, d.long_segptr, int32_t(h->long_rows.size()), part, nxt, k, koff, p.kc, scale_in,
