@@ -1126,13 +1126,20 @@ static int make_plan(const arrow_handle_s* h, int64_t k, int x_dtype, int flags,
     const int64_t most = int64_t(sm) * std::min(h->tune.ctas_per_sm, cap);
     // With the rescale every CTA also ends with FP64 sums of its columns (about two FP64 operations per clock
     // and SM), which more CTAs repeat: narrow rows share tiles up to one CTA per SM only, wide ones
-    // (whose rows are longer chains and whose sums take fewer steps) up to two, or three where that
-    // gives every tile two.  10 iterations in us, up to all resident CTAs / no sharing / this rule: 150^2
-    // grid (88 tiles) k = 32 BF16 168 / 118 / 118, k = 128 BF16 233 / 178 / 158; 250 x 200 grid (196 tiles)
-    // k = 128 FP32 276 / 264 / 219.
+    // (longer chains, sums of fewer steps) up to two, or three where that gives every tile two (four with
+    // 16 lanes of FP32).  10 iterations in us, up to all resident CTAs / no sharing / this rule: 150^2 grid
+    // (88 tiles) k = 32 BF16 168 / 118 / 118, k = 128 BF16 233 / 178 / 158; 250 x 200 grid (196 tiles) k = 128 FP32
+    // 276 / 264 / 219; random-geometric 60,007 rows (264 tiles) k = 128 FP32 355 / 308 / 308, k = 256 BF16 438 / 380 /
+    // 380; R-MAT 16 (275 tiles) k = 64 FP32 666 / 695 / 666.  Rows of under 2.5 entries leave a wide CTA with few
+    // gathers to wait for, so they share up to all resident CTAs: 60,000 rows of 0-3 entries (235 tiles) k = 256
+    // FP32 445 / 587; of 0-6 entries 634 / 633.
     int64_t share_most = most;
-    if (flags & ARROW_RESCALE)
-        share_most = std::min<int64_t>(most, p.T < 16 ? sm : std::max<int64_t>(2 * sm, std::min<int64_t>(3 * sm, 2 * n_tiles)));
+    if (flags & ARROW_RESCALE) {
+        if (p.T < 16) share_most = sm;
+        else if (p.T == 16 || 2 * int64_t(h->f_col.size()) >= 5 * h->n)
+            share_most = std::max<int64_t>(2 * sm, std::min<int64_t>((p.T == 16 && p.V == 4 ? 4 : 3) * sm, 2 * n_tiles));
+        share_most = std::min(share_most, most);
+    }
     p.parts = share ? row_parts(n_tiles, share_most, h->tune.tile_rows, 256 / p.T) : 1;
     p.rows_grid = int(std::max<int64_t>(1, std::min<int64_t>(n_tiles * p.parts, most)));
     const int64_t n_long = int64_t(h->long_rows.size());
