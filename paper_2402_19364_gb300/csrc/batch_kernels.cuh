@@ -118,11 +118,12 @@ __global__ void __launch_bounds__(256, kBatchMinBlocks) arrow_batch_rows_kernel(
         for (int b = 0; b < kStages; ++b)
             if (int64_t(blockIdx.x) + b * G < U) issue(blockIdx.x + b * G, b);
     pdl_wait();
-    // The next kernel comes in early where every CTA of this one has at most one unit.  Persistent CTAs hold
-    // their places longer on some SMs than on others, and a next rows kernel that came in beside them
-    // was placed as unevenly: 3 random-geometric matrices (k = 8, 16, 32 BF16), 10 iterations in one graph 136 us
-    // with an early trigger, 113 without (131 before launches overlapped); small ones, 25 of them, 146 / 148.
-    if (U <= G) pdl_launch();
+    // The next kernel comes in early where every CTA of this one has at most one unit, or many.  With a few,
+    // some CTAs hold their places much longer than others, and a next rows kernel that came in beside
+    // them was placed as unevenly: 3 random-geometric matrices (k = 8, 16, 32 BF16), 10 iterations in one graph 136
+    // us with an early trigger, 113 without (131 before launches overlapped).  25 small ones 146 / 148;
+    // 24 of up to 1 M rows (21 units a CTA) 1985 / 1996; 25 of up to 200,000 (6 units) 585 / 583.
+    if (U <= G || U >= 8 * G) pdl_launch();
     int i = 0;
     for (int64_t w = blockIdx.x; w < U; w += G, ++i) {
         const int b = i % kStages;
