@@ -213,13 +213,16 @@ __global__ void __launch_bounds__(256, RESCALE ? ARROW_ROWS_MIN_BLOCKS_RESCALE :
         const int32_t* scol = reinterpret_cast<const int32_t*>(buf + a.rp_bytes) + (e0 & 3);
         const TV* sval = reinterpret_cast<const TV*>(buf + a.rp_bytes + a.col_bytes) + (e0 & (VE - 1));
         const int nrows = r1 - r0;
-        // the next row's descriptor is read a row ahead (the word after the last is never used)
+        // the next row's descriptor is read a row ahead (the word after the last is never used); row pointers
+        // are not: with one ahead the BF16 kernel was up to 8 % slower (100,003 rows of 25 entries, k = 1024,
+        // 10 iterations 3363 us against 3107), with both ahead the FP32 rescale (1908 -> 2044)
         const int step = TEAMS * a.parts;
-        uint32_t dn = sdesc[min(q0, nrows)];
+        uint32_t dn = IN_ORDER ? 0 : sdesc[min(q0, nrows)];
         for (int q = q0; q < nrows; q += step) {
+            if (IN_ORDER) dn = sdesc[q];
             const RowDesc rd = IN_ORDER ? RowDesc{int(dn) - e0, q, int(sdesc[q + 1] - dn)}
                                         : row_desc_unpack(dn, a.long_rowptr, r0);
-            dn = sdesc[min(q + step, nrows)];
+            if (!IN_ORDER) dn = sdesc[min(q + step, nrows)];
             const int s = rd.start, e = rd.start + rd.len;
             // (with the rescale the permute-out is never folded in)
             const int64_t yr0 = !RESCALE && a.out_idx ? __ldg(a.out_idx + r0 + rd.row) : r0 + rd.row;
@@ -1188,8 +1191,8 @@ static int sigma_of(int flags) {
 // the L1 hits that neighbouring rows' gathers share; but long rows first keep the end of a tile short
 // where lengths are uneven.  So such rows come in row order, from the row pointers, where the
 // lengths are even (arrow_handle_s::even_rows: mean square at most 1.2 times the squared mean).  10
-// iterations in us, by length / in row order: random-geometric 100,003 rows (ratio 1.10) k = 256 FP32 870 / 782,
-// k = 512 BF16 908 / 820; 317 x 211 grid (1.00) k = 256 FP32 436 / 425; 20,000 rows of 0-60 entries (1.35)
+// iterations in us, by length / in row order: random-geometric 100,003 rows (ratio 1.10) k = 256 FP32 844 / 759,
+// k = 512 BF16 898 / 798; 317 x 211 grid (1.00) k = 256 FP32 414 / 412; 20,000 rows of 0-60 entries (1.35)
 // k = 256 FP32 437 / 466; R-MAT 15 (3.4) 1192 / 1265.
 static bool rows_in_order(const arrow_handle_s* h, const Plan& p) { return p.T == 32 && h->even_rows; }
 
